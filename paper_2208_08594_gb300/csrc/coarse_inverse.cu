@@ -1,0 +1,1116 @@
+// Dense FP64 inverse of the coarsest AMG matrix (Section 5: a direct solver), by blocked
+// in-place Gauss-Jordan with partial pivoting.  One step takes the kP = 96 columns K:
+//   1. LU with partial pivoting of the rows k0..n-1 of a copy of those columns, in
+//      sub-panels of W columns by one thread-block cluster (lu_panel_kernel) with rank-W
+//      updates of the rest of the copy in between (lu_update_kernel);
+//   2. D = A_KK^-1 from the factors, one warp per column (diag_inverse_panel_kernel), and
+//      the panel's row exchanges applied to all columns of A (swap_slice_kernel);
+//   3. A_iK <- P_iK = -A_iK D for the rows outside K, A_KK <- D, and with T = A_K,: before
+//      the step, A_ij += P_iK T_j outside K and A_Kj = D T_j (slice_gemm_kernel).
+// Step 3 is 2 n^3 flops in all.  The FP64 pipes do 1.25 TFLOP/s on this part, so it runs on
+// the fifth-generation tensor cores instead, without losing precision: every FP64 operand
+// is scaled by a power of two per row of P (per column of T) and written as eight signed
+// radix-256 digits, integers that bf16 holds exactly.  The product of two digits is at most
+// 2^14, and the sum over 96 terms and the up to eight digit pairs (i, j) with the same i + j
+// at most 8 * 96 * 2^14 < 2^24, so every FP32 accumulator holds an exact integer.  The 36
+// pairs with i + j <= 9 are kept (seven digits lost accuracy where a row's entries differ
+// widely); an epilogue adds the eight sums in integer arithmetic and rounds when it adds
+// them to C.  Every instruction multiplies digit i of P by the digits 1..9-i of T side by
+// side (N = 32 (9 - i)), each into the accumulator columns of its i + j.
+//
+// One SETUP's inverse, before (rank-32 updates on the FP64 pipes, two launches per column)
+// and now: n = 2,048: 45 -> 13 ms, 4,231: 203 -> 36 ms, 5,867: 446 -> 62 ms, 9,836: 1,824 ->
+// 178 ms (21 TFLOP/s of FP64 arithmetic).  Errors against an extended-precision solve are
+// below the previous kernels' (9,836 rows: 7.5e-16 against 1.8e-15).
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "setup_kernels.h"
+
+namespace msp {
+
+namespace {
+
+namespace cg = cooperative_groups;
+
+constexpr int kP = 96;         // columns of a Gauss-Jordan step
+constexpr int kDigits = 8;     // radix-256 digits of an operand
+constexpr int kRowTile = 128;  // rows of a product tile (one MMA's M)
+constexpr int kColTile = 32;   // columns of a product tile
+constexpr int kKTiles = kP / kColTile;
+constexpr int kChunk = 16;     // columns of K per copy (one MMA's K)
+constexpr int kChunks = kP / kChunk;
+constexpr int kStages = 4;     // chunk buffers of a column tile's digits
+constexpr int kGroups = kDigits;  // sums of digit pairs with equal i + j = 2..9
+// bytes of one K chunk of a row tile's / column tile's digits (bf16, core matrices of 8
+// rows x 16 bytes; kc: 16-byte groups along K)
+constexpr int kSliceA = kRowTile * kChunk * 2;            // one digit of a row tile
+constexpr int kChunkA = kDigits * kSliceA;                // 32,768
+constexpr int kTileA = kChunks * kChunkA;                 // 196,608
+constexpr int kRowsB = kDigits * kColTile;                // digits side by side
+constexpr int kChunkB = kRowsB * kChunk * 2;              // 8,192
+constexpr int kTileB = kChunks * kChunkB;                 // 49,152
+constexpr int kZeroExp = -4000;                           // exponent of an all-zero row
+
+inline int launch_status() { return launch_check(__FILE__, __LINE__); }
+
+__device__ void raise_flag(DevFlags* f, int code, int index) {
+  if (atomicCAS(&f->code, MSP_OK, code) == MSP_OK) f->index = index;
+}
+
+// ------------------------------------------------------------------ digits
+// e with |x| < 2^e for every |x| <= amax; amax 0 -> kZeroExp; not finite -> a large
+// exponent, so that every product with the row is not finite either
+__device__ __forceinline__ int scale_exp(double amax) {
+  if (amax == 0.0) return kZeroExp;
+  const int e = (int)((__double_as_longlong(amax) >> 52) & 0x7ff);
+  if (e == 0x7ff) return 1 << 20;
+  return max(e - 1022, -900);  // entries below 2^-955 lose digits
+}
+
+// x / 2^e (below 1) as a signed 64-bit integer in units of 2^-63
+__device__ __forceinline__ long long scaled_int(double x, int e) {
+  if (e == kZeroExp) return 0;
+  if (e > 2000) return 1LL << 40;  // any nonzero value: the exponent makes it infinite
+  // 2^(63 - e) in two factors, both representable
+  const int h = (63 - e) / 2, k = 63 - e - h;
+  const double s0 = __longlong_as_double((long long)(h + 1023) << 52);
+  const double s1 = __longlong_as_double((long long)(k + 1023) << 52);
+  return __double2ll_rn(x * s0 * s1);
+}
+
+__device__ __forceinline__ unsigned bf16_of_int(int d) {  // exact for |d| <= 256
+  return __float_as_uint((float)d) >> 16;
+}
+
+// the digits of eight consecutive operands along K, packed eight bf16 per digit:
+// digit s (0 = most significant) to dst + s * stride
+__device__ __forceinline__ void store_digits8(const double (&x)[8], int e, char* dst,
+                                              size_t stride) {
+  long long v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = scaled_int(x[q], e);
+#pragma unroll
+  for (int s = kDigits - 1; s >= 0; --s) {
+    unsigned w[4];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      int d;
+      if (s > 0) {
+        d = (int)(((unsigned)v[q] + 128u) & 255u) - 128;
+        v[q] = (v[q] - d) >> 8;
+      } else {
+        d = (int)v[q];  // |v| <= 128
+      }
+      const unsigned h = bf16_of_int(d);
+      if (q & 1)
+        w[q / 2] |= h << 16;
+      else
+        w[q / 2] = h;
+    }
+    *reinterpret_cast<uint4*>(dst + (size_t)s * stride) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// Digits of the rows of a tile of 32 rows of A[:, k0..k0+96) (A padded: whole tiles exist),
+// and the row exponents.  With Y the rows [z0, z1) are taken as zeros, and Y (kP values a
+// row) receives A[:, k0..k0+96) with -I in the rows [z0, z1).
+__global__ void __launch_bounds__(256) slice_rows_kernel(int lda, int k0, int z0, int z1,
+                                                         const double* __restrict__ A,
+                                                         char* __restrict__ S,
+                                                         int* __restrict__ exps,
+                                                         double* __restrict__ Y) {
+  __shared__ double sh[32][kP + 1];
+  __shared__ int se[32];
+  const int r0 = blockIdx.x * 32;
+  for (int t = threadIdx.x; t < 32 * kP; t += 256) {
+    const int r = t / kP, q = t % kP, i = r0 + r;
+    const bool z = Y && i >= z0 && i < z1;
+    const double x = z ? 0.0 : A[(size_t)i * lda + k0 + q];
+    sh[r][q] = x;
+    if (Y) Y[(size_t)i * kP + q] = z ? (i - z0 == q ? -1.0 : 0.0) : x;
+  }
+  __syncthreads();
+  {
+    const int r = threadIdx.x / 8, l = threadIdx.x % 8;  // eight lanes per row
+    double m = 0.0;
+    bool bad = false;
+    for (int q = l; q < kP; q += 8) {
+      const double a = fabs(sh[r][q]);
+      bad |= !isfinite(a);
+      m = fmax(m, a);
+    }
+    if (bad) m = __longlong_as_double(0x7ff0000000000000LL);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o, 8));
+    if (l == 0) {
+      const int e = scale_exp(m);
+      se[r] = e;
+      exps[r0 + r] = e;
+    }
+  }
+  __syncthreads();
+  char* tile = S + (size_t)(r0 / kRowTile) * kTileA;
+  for (int t = threadIdx.x; t < 32 * (kP / 8); t += 256) {
+    const int r = t % 32, kcg = t / 32;
+    double x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = sh[r][kcg * 8 + q];
+    const int tr = (r0 + r) % kRowTile;
+    char* dst = tile + (size_t)(kcg / 2) * kChunkA + (kcg % 2) * (kRowTile / 8) * 128 +
+                (tr / 8) * 128 + (tr % 8) * 16;
+    store_digits8(x, se[r], dst, kSliceA);
+  }
+}
+
+// digit s of column c (of a tile of 32), 16-byte group kcg of K, in a column tile's image
+__device__ __forceinline__ char* digit_b(char* tile, int c, int kcg) {
+  return tile + (size_t)(kcg / 2) * kChunkB + (kcg % 2) * (kRowsB / 8) * 128 + (c / 8) * 128 +
+         (c % 8) * 16;
+}
+constexpr int kDigitStrideB = (kColTile / 8) * 128;
+
+// The panel's row exchanges on a tile of 32 columns of A, and the digits of the exchanged
+// rows K (T, for the tiles of K the block A_KK).  perm[0] = number of rows that change, then pairs
+// (destination, source); the K rows of T are read after the exchange.
+__global__ void __launch_bounds__(256) swap_slice_kernel(int lda, int k0, int kb,
+                                                         double* __restrict__ A,
+                                                         const int* __restrict__ perm,
+                                                         char* __restrict__ S,
+                                                         int* __restrict__ exps) {
+  extern __shared__ double swap_smem[];  // [2 kP][33]
+  double(*sh)[kColTile + 1] = reinterpret_cast<double(*)[kColTile + 1]>(swap_smem);
+  __shared__ int sd[2 * kP];
+  __shared__ double smax[8][kColTile];
+  __shared__ int se[kColTile];
+  const int ct = blockIdx.x, c0 = ct * kColTile;
+  const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
+  const int cnt = perm[0];
+  for (int t = w; t < cnt; t += 8) {
+    if (lane == 0) sd[t] = perm[1 + 2 * t];
+    sh[t][lane] = A[(size_t)perm[2 + 2 * t] * lda + c0 + lane];
+  }
+  __syncthreads();
+  for (int t = w; t < cnt; t += 8) A[(size_t)sd[t] * lda + c0 + lane] = sh[t][lane];
+  __syncthreads();  // the rows K below are read back by the block that wrote them
+  for (int q = w; q < kP; q += 8)
+    sh[q][lane] = q < kb ? A[(size_t)(k0 + q) * lda + c0 + lane] : 0.0;
+  __syncthreads();
+  double m = 0.0;
+  bool bad = false;
+  for (int q = w; q < kP; q += 8) {
+    const double a = fabs(sh[q][lane]);
+    bad |= !isfinite(a);
+    m = fmax(m, a);
+  }
+  smax[w][lane] = bad ? __longlong_as_double(0x7ff0000000000000LL) : m;
+  __syncthreads();
+  if (w == 0) {
+    for (int u = 1; u < 8; ++u) m = fmax(m, smax[u][lane]);
+    m = fmax(m, smax[0][lane]);
+    const int e = scale_exp(m);
+    se[lane] = e;
+    exps[c0 + lane] = e;
+  }
+  __syncthreads();
+  char* tile = S + (size_t)ct * kTileB;
+  for (int t = threadIdx.x; t < kColTile * (kP / 8); t += 256) {
+    const int c = t % kColTile, kcg = t / kColTile;
+    double x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = sh[kcg * 8 + q][c];
+    store_digits8(x, se[c], digit_b(tile, c, kcg), kDigitStrideB);
+  }
+}
+
+// ------------------------------------------------------------------ LU of the panel copy
+// X[i][c] = A[k0 + i][k0 + c] for the rows below k0, columns past kb zero
+__global__ void panel_copy_kernel(int m, int k0, int kb, int lda, const double* __restrict__ A,
+                                  double* __restrict__ X) {
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)m * kP;
+       t += (size_t)gridDim.x * blockDim.x) {
+    const int i = (int)(t / kP), c = (int)(t % kP);
+    X[t] = c < kb ? A[(size_t)(k0 + i) * lda + k0 + c] : 0.0;
+  }
+}
+
+// LU with partial pivoting (the first of equal largest entries wins) of the columns
+// [c0, c0 + w) of the panel copy X (m rows of kP), rows c0..m-1, by one cluster: thread t of
+// CTA c holds the rows c * rpc + t + r * blockDim, r < R, in registers, the columns still to
+// be factored first: after every step they move one place left and the step's multiplier
+// takes the last place, so that the loop over the columns stays a loop (unrolled, its
+// once-run code missed the instruction cache: 5.4 us a column at 4,231 rows) and nothing is
+// stored before it ends (the barrier's release would wait for the stores: 3.5 us).  A column costs one cluster barrier: the warp that holds a CTA's
+// best pivot candidate sends that row to every CTA (and the owner of row k the row to be
+// exchanged), so after the barrier every CTA has the pivot row; the slots alternate by the
+// parity of the column.  Bound by that chain of latencies and by the FP64 rate of the
+// cluster's SMs.  CTA 0 then
+// exchanges the rows of the panel's other columns and solves for the U rows of the columns
+// to the right.  piv[c0 + q] = row exchanged with row c0 + q.
+constexpr int kLuThreads = 512;
+constexpr int kMaxCluster = 16;
+
+__device__ __forceinline__ unsigned long long magnitude(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
+  return b > 0x7ff0000000000000ULL ? 0 : b;  // NaN is no candidate
+}
+// over the warp: the largest value, the smallest index among equal ones
+__device__ __forceinline__ void warp_best(unsigned long long& v, int& i) {
+  const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  i = (int)__reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? (unsigned)i : 0x7fffffffu);
+  v = ((unsigned long long)mh << 32) | ml;
+}
+
+template <int W, int R>
+__global__ void __launch_bounds__(kLuThreads) lu_panel_kernel(int m, int c0, int w, int kb, int rpc,
+                                                              double* __restrict__ X,
+                                                              int* __restrict__ piv, int k0,
+                                                              DevFlags* flags) {
+  __shared__ __align__(16) double cand[2][kMaxCluster][W + 2];  // every CTA's best row, 1 / pivot
+  __shared__ __align__(16) double rowk[2][W + 2];               // row k before the exchange
+  __shared__ __align__(16) double out[kLuThreads / kWarp][2][W + 2];  // a warp's rows to send
+  __shared__ unsigned long long cmag[2][kMaxCluster], wmag[2][kLuThreads / kWarp];
+  __shared__ int cidx[2][kMaxCluster], widx[2][kLuThreads / kWarp], spiv[W], slot[W];
+  __shared__ double xs[2 * W * kP];  // CTA 0: the rows that the exchanges move
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), nct = (int)cluster.num_blocks();
+  const int tid = threadIdx.x, lane = tid % kWarp, wid = tid / kWarp;
+  const int nw = (int)blockDim.x / kWarp;
+  const int base = c0 + rank * rpc;
+  int row[R];  // m: none
+  double a[R][W];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int q = tid + r * (int)blockDim.x;
+    row[r] = q < rpc && base + q < m ? base + q : m;
+#pragma unroll
+    for (int c = 0; c < W; ++c)
+      a[r][c] = row[r] < m && c < w ? X[(size_t)row[r] * kP + c0 + c] : 0.0;
+  }
+  cluster.sync();  // every CTA's shared memory is live before it is written remotely
+  // the row held by the thread with `own` (at most one of the block, any of its R rows) to
+  // the same place in every CTA: staged by the thread, sent by its warp, 16 bytes a lane
+  auto send = [&](bool own, int r, int which, double* dst) {
+    const unsigned has = __ballot_sync(0xffffffffu, own);
+    if (!has) return;
+    if (own) {
+#pragma unroll
+      for (int rr = 0; rr < R; ++rr)
+        if (rr == r) {
+          // the reciprocal is taken here, by one warp: by every warp after the barrier its
+          // dozen FP64 instructions would fill the pipe
+          if (which == 0) out[wid][0][W] = 1.0 / a[rr][0];
+#pragma unroll
+          for (int c = 0; c < W; ++c) out[wid][which][c] = a[rr][c];
+        }
+    }
+    __syncwarp();
+    constexpr int kPairs = W / 2 + 1;
+    for (int t = lane; t < nct * kPairs; t += kWarp) {
+      const int d = t / kPairs, c = t % kPairs;
+      reinterpret_cast<double2*>(cluster.map_shared_rank(dst, d))[c] =
+          reinterpret_cast<const double2*>(out[wid][which])[c];
+    }
+  };
+#pragma unroll 1
+  for (int k = 0; k < w; ++k) {
+    const int par = k & 1, kr = c0 + k;  // row of the diagonal
+    // best candidate among the rows >= kr (magnitudes compared as integers, 0: none)
+    unsigned long long best = 0;
+    int bi = m;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const unsigned long long v = row[r] >= kr && row[r] < m ? magnitude(a[r][0]) : 0;
+      if (v > best) {
+        best = v;
+        bi = row[r];
+      }
+    }
+    warp_best(best, bi);
+    if (lane == 0) {
+      wmag[par][wid] = best;
+      widx[par][wid] = bi;
+    }
+    __syncthreads();
+    best = lane < nw ? wmag[par][lane] : 0;
+    bi = lane < nw ? widx[par][lane] : m;
+    warp_best(best, bi);
+    bool mine = false, diag = false;
+    int rm = 0, rd = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (best && row[r] == bi) {
+        mine = true;
+        rm = r;
+      }
+      if (row[r] == kr) {
+        diag = true;
+        rd = r;
+      }
+    }
+    send(mine, rm, 0, cand[par][rank]);
+    send(diag, rd, 1, rowk[par]);
+    if (wid == 0 && lane < nct) {
+      cluster.map_shared_rank(&cmag[par][rank], lane)[0] = best;
+      cluster.map_shared_rank(&cidx[par][rank], lane)[0] = bi;
+    }
+    cluster.sync();
+    unsigned long long pb = lane < nct ? cmag[par][lane] : 0;
+    int pi = lane < nct ? cidx[par][lane] : m;
+    const unsigned long long pmine = pb;
+    const int imine = pi;
+    warp_best(pb, pi);
+    const int pr = __ffs(__ballot_sync(0xffffffffu, pmine == pb && imine == pi)) - 1;
+    const bool ok = pb != 0;  // no usable pivot: the column is left out, the flag raised
+    if (!ok) pi = kr;
+    const double* up = ok ? cand[par][pr] : rowk[par];
+    double u[W];
+#pragma unroll
+    for (int c = 0; c < W; c += 2) {
+      const double2 v = *reinterpret_cast<const double2*>(up + c);
+      u[c] = v.x;
+      u[c + 1] = v.y;
+    }
+    if (tid == 0) {
+      spiv[k] = pi;
+      if (rank == 0) {
+        piv[c0 + k] = pi;
+        if (!ok) raise_flag(flags, MSP_ERR_SINGULAR_BLOCK, k0 + kr);
+      }
+    }
+    const double inv = ok ? up[W] : 0.0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (row[r] == pi && pi != kr) {  // the row exchanged away from the diagonal
+#pragma unroll
+        for (int c = 0; c < W; ++c) a[r][c] = rowk[par][c];
+      }
+      if (row[r] == kr) {
+#pragma unroll
+        for (int c = 0; c < W; ++c) a[r][c] = u[c];
+      } else if (row[r] > kr && row[r] < m) {
+        const double l = a[r][0] * inv;
+#pragma unroll
+        for (int g = 0; g < W; g += 4) {
+          if (g + k < W) {  // some of these places still hold columns to be factored
+#pragma unroll
+            for (int c = g; c < g + 4 && c < W; ++c)
+              if (c > 0) a[r][c - 1] = c + k < W ? fma(-l, u[c], a[r][c]) : a[r][c];
+          } else {
+#pragma unroll
+            for (int c = g; c < g + 4 && c < W; ++c)
+              if (c > 0) a[r][c - 1] = a[r][c];
+          }
+        }
+        a[r][W - 1] = l;
+      }
+    }
+  }
+  // place c of a row holds column (c + steps) % W; a row of U stopped at its own step
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (row[r] < m) {
+      const int steps = min(row[r] - c0, w);
+      double* x = X + (size_t)row[r] * kP + c0;
+#pragma unroll
+      for (int c = 0; c < W; ++c) {
+        const int col = (c + steps) % W;
+        if (col < w) x[col] = a[r][c];
+      }
+    }
+  cluster.sync();  // remote writes and reads are done; the factored columns are stored
+  if (rank != 0) return;
+  // the other columns: rows c0 + q <-> spiv[q], slots 0..w-1 the rows c0.., slot w + q the
+  // pivot row of step q unless it is one of those or an earlier step's
+  if (tid < w) {
+    const int p = spiv[tid];
+    int s = W + tid;
+    if (p < c0 + w) {
+      s = p - c0;
+    } else {
+      for (int q = tid - 1; q >= 0; --q)
+        if (spiv[q] == p) s = W + q;
+    }
+    slot[tid] = s;
+  }
+  __syncthreads();
+  for (int t = tid; t < 2 * W * kP; t += blockDim.x) {
+    const int s = t / kP, c = t % kP;
+    const int q = s % W;
+    if (q >= w || (s >= W && slot[q] != s)) continue;
+    xs[t] = X[(size_t)(s < W ? c0 + q : spiv[q]) * kP + c];
+  }
+  __syncthreads();
+  if (tid < kP && (tid < c0 || tid >= c0 + w)) {
+    for (int q = 0; q < w; ++q) {
+      const int s = slot[q];
+      if (s != q) {
+        const double t = xs[q * kP + tid];
+        xs[q * kP + tid] = xs[s * kP + tid];
+        xs[s * kP + tid] = t;
+      }
+    }
+  }
+  __syncthreads();
+  {
+    if (tid >= c0 + w && tid < kb) {
+      double y[W];
+#pragma unroll
+      for (int q = 0; q < W; ++q) y[q] = q < w ? xs[q * kP + tid] : 0.0;
+#pragma unroll
+      for (int k = 0; k < W; ++k)
+        if (k < w) {
+#pragma unroll
+          for (int q = k + 1; q < W; ++q)
+            if (q < w) y[q] = fma(-xs[q * kP + c0 + k], y[k], y[q]);
+        }
+#pragma unroll
+      for (int q = 0; q < W; ++q)
+        if (q < w) xs[q * kP + tid] = y[q];
+    }
+  }
+  __syncthreads();
+  for (int t = tid; t < 2 * W * kP; t += blockDim.x) {
+    const int s = t / kP, c = t % kP;
+    const int q = s % W;
+    if (q >= w || (s >= W && slot[q] != s)) continue;
+    X[(size_t)(s < W ? c0 + q : spiv[q]) * kP + c] = xs[t];
+  }
+}
+
+// X[i][j] -= sum_q X[i][c0 + q] X[c0 + q][j] for the rows below c0 + w and the columns right
+// of it: 16 rows per block (64 left most SMs without a block on the usual 2,000 to 10,000
+// rows: 27 us a launch at 4,231), the multipliers and the U rows staged in shared memory
+constexpr int kUpdRows = 16;
+template <int W>
+__global__ void __launch_bounds__(256) lu_update_kernel(int m, int c0, int w, int kb,
+                                                        double* __restrict__ X) {
+  __shared__ double sl[kUpdRows][W + 1];
+  __shared__ double su[W][kP];
+  const int j0 = c0 + w, nj = kb - j0, r0 = c0 + w + blockIdx.x * kUpdRows;
+  for (int t = threadIdx.x; t < kUpdRows * W; t += 256) {
+    const int r = t / W, q = t % W;
+    sl[r][q] = (r0 + r < m && q < w) ? X[(size_t)(r0 + r) * kP + c0 + q] : 0.0;
+  }
+  for (int t = threadIdx.x; t < W * kP; t += 256) {
+    const int q = t / kP, j = t % kP;
+    su[q][j] = (q < w && j < nj) ? X[(size_t)(c0 + q) * kP + j0 + j] : 0.0;
+  }
+  __syncthreads();
+  const int tx = threadIdx.x % 16, i = r0 + threadIdx.x / 16;
+  if (i >= m) return;
+  const double* l = sl[threadIdx.x / 16];
+  for (int j = tx; j < nj; j += 16) {
+    double a = X[(size_t)i * kP + j0 + j];
+#pragma unroll
+    for (int q = 0; q < W; ++q) a = fma(-l[q], su[q][j], a);
+    X[(size_t)i * kP + j0 + j] = a;
+  }
+}
+
+// D = A_KK^-1 (rows K exchanged) from the factors in X: one warp per column solves
+// L y = e_j, U x = y by columns (lane l owns the rows l, l + 32, l + 64; a step is a
+// broadcast and up to three FMAs).  D is stored (kP x kP, zero past kb) and so are its
+// digits (as a T operand) with their exponents.  The last block composes the exchanges
+// into the list of rows that change (perm) for all columns of A.
+constexpr int kDiagWarps = 4;
+__global__ void __launch_bounds__(kDiagWarps * kWarp) diag_inverse_panel_kernel(
+    int k0, int kb, const double* __restrict__ X, const int* __restrict__ piv,
+    double* __restrict__ D, char* __restrict__ S, int* __restrict__ exps,
+    int* __restrict__ perm, int* __restrict__ piv_out) {
+  extern __shared__ double sf[];  // kP x (kP + 1) factors, then kP reciprocal pivots
+  if (blockIdx.x == gridDim.x - 1) {
+    // exchanges in order on a small list: slot q < kb is row k0 + q, slot kb + q the pivot
+    // row of step q when it lies below the block (the first step that names it)
+    __shared__ int row[2 * kP], cur[2 * kP], sl[kP], sp[kP];
+    for (int q = threadIdx.x; q < kb; q += blockDim.x) sp[q] = piv[q];
+    __syncthreads();
+    for (int q = threadIdx.x; q < kb; q += blockDim.x) {
+      const int p = sp[q];
+      int s = kb + q;
+      if (p < kb) {
+        s = p;
+      } else {
+        for (int r = q - 1; r >= 0; --r)
+          if (sp[r] == p) s = kb + r;
+      }
+      sl[q] = s;
+      row[q] = k0 + q;
+      row[kb + q] = s == kb + q ? k0 + p : -1;
+      piv_out[k0 + q] = k0 + p;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < 2 * kb; t += blockDim.x) cur[t] = t;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int q = 0; q < kb; ++q) {
+        const int s = sl[q], a = cur[q];
+        cur[q] = cur[s];
+        cur[s] = a;
+      }
+    __syncthreads();
+    if (threadIdx.x < kWarp) {  // compacted by one warp
+      int cnt = 0;
+      for (int t0 = 0; t0 < 2 * kb; t0 += kWarp) {
+        const int t = t0 + threadIdx.x;
+        const bool ch = t < 2 * kb && row[t] >= 0 && cur[t] != t;
+        const unsigned b = __ballot_sync(0xffffffffu, ch);
+        const int at = cnt + __popc(b & ((1u << threadIdx.x) - 1u));
+        if (ch) {
+          perm[1 + 2 * at] = row[t];
+          perm[2 + 2 * at] = row[cur[t]];
+        }
+        cnt += __popc(b);
+      }
+      if (threadIdx.x == 0) perm[0] = cnt;
+    }
+    return;
+  }
+  constexpr int ld = kP + 1;
+  double* rd = sf + kP * ld;
+#pragma unroll 8
+  for (int t = threadIdx.x; t < kP * kP; t += kDiagWarps * kWarp) {
+    const int r = t / kP, c = t % kP;
+    sf[r * ld + c] = (r < kb && c < kb) ? X[(size_t)r * kP + c] : 0.0;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < kP; q += blockDim.x) {
+    const double d = sf[q * ld + q];
+    rd[q] = d != 0.0 ? 1.0 / d : 0.0;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x % kWarp;
+  const int j = blockIdx.x * kDiagWarps + threadIdx.x / kWarp;
+  double y[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) y[a] = (lane + 32 * a == j && j < kb) ? 1.0 : 0.0;
+#pragma unroll 4
+  for (int k = j & ~3; k < kb; ++k) {  // rows above j stay zero
+    const double mine = k < 32 ? y[0] : (k < 64 ? y[1] : y[2]);
+    const double yk = __shfl_sync(0xffffffffu, mine, k & 31);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      if (lane + 32 * a > k) y[a] = fma(-sf[(lane + 32 * a) * ld + k], yk, y[a]);
+  }
+#pragma unroll 4
+  for (int k = kb - 1; k >= 0; --k) {
+    const double mine = (k < 32 ? y[0] : (k < 64 ? y[1] : y[2])) * rd[k];
+    const double xk = __shfl_sync(0xffffffffu, mine, k & 31);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if (lane + 32 * a < k)
+        y[a] = fma(-sf[(lane + 32 * a) * ld + k], xk, y[a]);
+      else if (lane + 32 * a == k)
+        y[a] = xk;
+    }
+  }
+  double m = 0.0;
+  bool bad = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (lane + 32 * a >= kb || j >= kb) y[a] = 0.0;
+    bad |= !isfinite(y[a]);
+    m = fmax(m, fabs(y[a]));
+    D[(size_t)(lane + 32 * a) * kP + j] = y[a];
+  }
+  if (bad) m = __longlong_as_double(0x7ff0000000000000LL);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int e = scale_exp(m);
+  if (lane == 0) exps[j] = e;
+  char* tile = S + (size_t)(j / kColTile) * kTileB;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int q = lane + 32 * a;
+    long long v = scaled_int(y[a], e);
+    char* dst = digit_b(tile, j % kColTile, q / 8) + (q % 8) * 2;
+    for (int s = kDigits - 1; s >= 0; --s) {
+      int d = (int)v;
+      if (s > 0) {
+        d = (int)(((unsigned)v + 128u) & 255u) - 128;
+        v = (v - d) >> 8;
+      }
+      *reinterpret_cast<unsigned short*>(dst + (size_t)s * kDigitStrideB) =
+          (unsigned short)bf16_of_int(d);
+    }
+  }
+}
+
+// ------------------------------------------------------------------ the products
+__device__ __forceinline__ unsigned smem_u32(const void* p) {
+  return (unsigned)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// Wait for the phase of the given parity, with a limit; false (and the block's stop word
+// set) when the limit runs out or another warp has stopped.
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* stop) {
+  for (int it = 0; it < (1 << 20); ++it) {
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (*stop) return false;
+  }
+  *stop = 1;
+  return false;
+}
+__device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes,
+                                          unsigned bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(dst),
+      "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(bar)
+      : "memory");
+}
+// shared-memory matrix descriptor: K-major, no swizzle, core matrices of 8 rows x 16 bytes;
+// lbo: bytes between core matrices along K, sbo: along the rows
+__device__ __forceinline__ unsigned long long mat_desc(unsigned addr, unsigned lbo, unsigned sbo) {
+  return (unsigned long long)((addr & 0x3ffffu) >> 4) | ((unsigned long long)(lbo >> 4) << 16) |
+         ((unsigned long long)(sbo >> 4) << 32) | (1ULL << 46);
+}
+// D (f32, TMEM) (+)= A (bf16) B (bf16)^T, M = 128, N = n, K = 16
+__device__ __forceinline__ void mma_bf16(unsigned d, unsigned long long a, unsigned long long b,
+                                         unsigned n, bool accumulate) {
+  const unsigned idesc =
+      (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((unsigned)(kRowTile >> 4) << 24);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate ? 1u : 0u)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit(unsigned bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(unsigned addr, unsigned (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(addr));
+}
+
+// c + sign 2^e sum_m S_m 2^(8 (9 - m)), m = 2..9, S_m exact integers below 2^24
+__device__ __forceinline__ double add_digits(const float (&S)[kGroups], int e, double sign,
+                                             double c) {
+  // two exact 64-bit integers, |lo| < 2^49 and |hi| < 2^49; the sum is hi 2^32 + lo
+  const int s2 = __float2int_rn(S[0]), s3 = __float2int_rn(S[1]), s4 = __float2int_rn(S[2]);
+  const int s5 = __float2int_rn(S[3]), s6 = __float2int_rn(S[4]), s7 = __float2int_rn(S[5]);
+  const int s8 = __float2int_rn(S[6]), s9 = __float2int_rn(S[7]);
+  const long long hi =
+      (long long)s2 * 16777216 + ((long long)s3 * 65536 + ((long long)s4 * 256 + s5));
+  const long long lo =
+      (long long)s6 * 16777216 + ((long long)s7 * 65536 + ((long long)s8 * 256 + s9));
+  // An integer below 2^51 added to the bits of M = 1.5 * 2^52 is the double M + integer.
+  // The low word is used as it is, M too large, and M = 1.5 * 2^20 * 2^32 is taken from the
+  // high word instead: three FP64 operations an element (the FP64 pipe bounds the epilogue).
+  const double dh =
+      __longlong_as_double(0x4338000000000000LL + (hi - 1572864)) - 6755399441055744.0;
+  const double dl = __longlong_as_double(0x4338000000000000LL + lo);
+  const int be = min(max(e + 1023, 0), 0x7ff), bh = min(max(e + 1055, 0), 0x7ff);
+  const long long sg = __double_as_longlong(sign) & (1LL << 63);
+  const double fl = __longlong_as_double(((long long)be << 52) | sg);
+  const double fh = __longlong_as_double(((long long)bh << 52) | sg);
+  return fma(dl, fl, fma(dh, fh, c));
+}
+
+// One product of a step on the tiles (128 x 32) of C (leading dimension ldc), V = SA SB:
+//   kUpdate: C = A, the columns outside K (kt0: the first tile of K, 3 tiles left out):
+//            C += V, or C = V for the rows K;
+//   kFirst:  C = the columns K: C = -V, or D for the rows K;
+//   kResid:  C += V;  kCorrect: C -= V (both on 96 columns).
+enum Product { kUpdate, kFirst, kResid, kCorrect };
+// Persistent blocks, each a contiguous run of tiles in row-major tile order; the digits of a
+// row tile (192 KB) stay in shared memory while the column tiles' digits (48 KB) stream
+// through four buffers of 16 columns of K, so L2 is read once per tile.  One warp copies, one thread of
+// another issues the MMAs (48 per tile, into one of two TMEM buffers of 256 columns), sixteen
+// warps turn the previous tile's accumulators into FP64 and update A.
+constexpr int kEpiWarps = 16;
+constexpr int kGemmThreads = (kEpiWarps + 2) * kWarp;
+constexpr int kEpiCols = kColTile / (kEpiWarps / 4);  // columns of a tile per epilogue warp
+constexpr size_t kGemmSmem = kTileA + kStages * kChunkB + 512;
+template <Product kMode>
+__global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
+    int ldc, int k0, int kb, int nrt, int nct, int kt0, double* __restrict__ C,
+    const char* __restrict__ SA, const int* __restrict__ ea, const char* __restrict__ SB,
+    const int* __restrict__ eb, const double* __restrict__ D, DevFlags* flags) {
+  extern __shared__ __align__(128) char sm[];
+  __shared__ __align__(8) unsigned long long bars[1 + 2 * kStages + 5];
+  __shared__ unsigned s_tmem;
+  __shared__ volatile int s_stop;
+  const int wid = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
+  const unsigned sbase = (smem_u32(sm) + 127u) & ~127u;
+  const unsigned sA = sbase, sB = sbase + kTileA;
+  const unsigned b_a = smem_u32(&bars[0]);
+  const unsigned b_full = smem_u32(&bars[1]), b_empty = smem_u32(&bars[1 + kStages]);
+  const unsigned b_tfull = smem_u32(&bars[1 + 2 * kStages]), b_tempty = b_tfull + 16;
+  const unsigned b_end = b_tempty + 16;  // used only after a stop
+  const long long total = (long long)nrt * nct;
+  const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
+  if (threadIdx.x == 0) {
+    s_stop = 0;
+    mbar_init(b_a, 1);
+    mbar_init(b_end, 1);
+    for (int c = 0; c < kStages; ++c) {
+      mbar_init(b_full + 8 * c, 1);
+      mbar_init(b_empty + 8 * c, 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(b_tfull + 8 * b, 1);
+      mbar_init(b_tempty + 8 * b, kEpiWarps);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (wid == kEpiWarps + 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                     smem_u32(&s_tmem))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem = s_tmem;
+
+  if (wid == kEpiWarps) {
+    if (lane == 0) {
+      int prev = -1;
+      unsigned g = 0;  // chunks so far: buffer g % kStages, its use g / kStages
+      bool run = true;
+      for (long long t = t0; t < t1 && run; ++t) {
+        const int rt = (int)(t / nct), q = (int)(t % nct);
+        const int ct = kMode != kUpdate ? q : q + (q >= kt0 ? kKTiles : 0);
+        if (rt != prev) {
+          // the previous row tile's digits are free once its last chunk has been used
+          if (g > 0)
+            run = mbar_wait(b_empty + 8 * ((g - 1) % kStages), ((g - 1) / kStages) & 1, &s_stop);
+          if (!run) break;
+          mbar_expect(b_a, kTileA);
+          for (int c = 0; c < kChunks; ++c)
+            bulk_load(sA + c * kChunkA, SA + (size_t)rt * kTileA + (size_t)c * kChunkA, kChunkA, b_a);
+          prev = rt;
+        }
+        for (int c = 0; c < kChunks && run; ++c, ++g) {
+          const unsigned st = g % kStages;
+          if (g >= kStages) run = mbar_wait(b_empty + 8 * st, ((g / kStages) - 1) & 1, &s_stop);
+          if (!run) break;
+          mbar_expect(b_full + 8 * st, kChunkB);
+          bulk_load(sB + st * kChunkB, SB + (size_t)ct * kTileB + (size_t)c * kChunkB, kChunkB,
+                    b_full + 8 * st);
+        }
+      }
+    }
+  } else if (wid == kEpiWarps + 1) {
+    if (lane == 0) {
+      int prev = -1;
+      unsigned it = 0, na = 0, g = 0;
+      bool run = true;
+      for (long long t = t0; t < t1 && run; ++t, ++it) {
+        const int rt = (int)(t / nct);
+        if (rt != prev) {
+          run = mbar_wait(b_a, na & 1, &s_stop);
+          ++na;
+          prev = rt;
+        }
+        const unsigned buf = it & 1;
+        if (run && it >= 2) run = mbar_wait(b_tempty + 8 * buf, ((it >> 1) - 1) & 1, &s_stop);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int c = 0; c < kChunks && run; ++c, ++g) {
+          const unsigned st = g % kStages;
+          run = mbar_wait(b_full + 8 * st, (g / kStages) & 1, &s_stop);
+          if (!run) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const unsigned long long db = mat_desc(sB + st * kChunkB, (kRowsB / 8) * 128, 128);
+          // digit i of P with the digits 0..7-i of T; digit 0 of the first chunk starts the
+          // eight sums
+#pragma unroll
+          for (int i = 0; i < kDigits; ++i)
+            mma_bf16(tmem + buf * 256 + i * kColTile,
+                     mat_desc(sA + c * kChunkA + i * kSliceA, (kRowTile / 8) * 128, 128), db,
+                     kColTile * (kDigits - i), c > 0 || i > 0);
+          mma_commit(b_empty + 8 * st);
+        }
+        if (run) mma_commit(b_tfull + 8 * buf);
+      }
+      // every MMA issued here ends before the accumulators and the buffers go away: the
+      // epilogue warps wait for all of them, and after a stop this waits for a commit
+      if (!run) {
+        volatile int never = 0;
+        mma_commit(b_end);
+        mbar_wait(b_end, 0, &never);
+      }
+    }
+  } else {
+    const int quad = wid & 3, part = wid >> 2;  // a warp reads the TMEM lanes of its quadrant
+    constexpr double sign = kMode == kFirst || kMode == kCorrect ? -1.0 : 1.0;
+    // what a tile's C starts from: the rows' and columns' values, loaded one tile ahead
+    auto load_c = [&](long long t, double (&cv)[kEpiCols]) {
+      const int rt = (int)(t / nct), q = (int)(t % nct);
+      const int ct = kMode != kUpdate ? q : q + (q >= kt0 ? kKTiles : 0);
+      const int i = rt * kRowTile + quad * 32 + lane;
+      const bool in_k = i >= k0 && i < k0 + kb;
+      const int cb = ct * kColTile + part * kEpiCols;
+      const double* src = kMode == kFirst ? D + (size_t)(i - k0) * kP + cb
+                                          : C + (size_t)i * ldc + cb;
+      const bool use = kMode == kFirst ? in_k : kMode != kUpdate || !in_k;
+#pragma unroll
+      for (int p = 0; p < kEpiCols / 2; ++p) {
+        const double2 v = use ? *reinterpret_cast<const double2*>(src + 2 * p)
+                              : make_double2(0.0, 0.0);
+        cv[2 * p] = v.x;
+        cv[2 * p + 1] = v.y;
+      }
+    };
+    unsigned it = 0;
+    double cn[kEpiCols];
+    if (t0 < t1) load_c(t0, cn);
+    for (long long t = t0; t < t1; ++t, ++it) {
+      const int rt = (int)(t / nct), q = (int)(t % nct);
+      const int ct = kMode != kUpdate ? q : q + (q >= kt0 ? kKTiles : 0);
+      const int i = rt * kRowTile + quad * 32 + lane;
+      const bool in_k = i >= k0 && i < k0 + kb;
+      const int cb = ct * kColTile + part * kEpiCols;
+      double* crow = C + (size_t)i * ldc + cb;
+      double cv[kEpiCols];
+#pragma unroll
+      for (int p = 0; p < kEpiCols; ++p) cv[p] = cn[p];
+      int ev[kEpiCols];  // exponents of row + column
+      const int eai = __ldg(ea + i) - 70;
+#pragma unroll
+      for (int c = 0; c < kEpiCols; c += 4) {
+        const int4 v = __ldg(reinterpret_cast<const int4*>(eb + cb + c));
+        ev[c] = v.x + eai;
+        ev[c + 1] = v.y + eai;
+        ev[c + 2] = v.z + eai;
+        ev[c + 3] = v.w + eai;
+      }
+      if (t + 1 < t1) load_c(t + 1, cn);
+      const unsigned buf = it & 1;
+      const bool run = mbar_wait(b_tfull + 8 * buf, (it >> 1) & 1, &s_stop);
+      if (!__all_sync(0xffffffffu, run)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      static_assert(kEpiCols == 8, "one load of eight columns per group");
+      unsigned r[kGroups][8];
+#pragma unroll
+      for (int m = 0; m < kGroups; ++m)
+        tmem_ld8(tmem + ((unsigned)(quad * 32) << 16) + buf * 256 + m * kColTile + part * kEpiCols,
+                 r[m]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      if (lane == 0) mbar_arrive(b_tempty + 8 * buf);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        float S[kGroups];
+#pragma unroll
+        for (int m = 0; m < kGroups; ++m) S[m] = __uint_as_float(r[m][c]);
+        const double v = add_digits(S, ev[c], sign, cv[c]);
+        if (kMode != kFirst || !in_k) cv[c] = v;
+      }
+#pragma unroll
+      for (int p = 0; p < kEpiCols / 2; ++p)
+        *reinterpret_cast<double2*>(crow + 2 * p) = make_double2(cv[2 * p], cv[2 * p + 1]);
+    }
+  }
+  __syncthreads();
+  if (s_stop) {
+    // a wait ran out: the copies in flight land before the block (and its shared memory)
+    // goes away; the last expected phase of every chunk is waited for, with a limit
+    if (threadIdx.x == 0) {
+      raise_flag(flags, MSP_ERR_TIMEOUT, blockIdx.x);
+      volatile int never = 0;
+      for (int par = 0; par < 2; ++par) {
+        mbar_wait(b_a, par, &never);
+        for (int c = 0; c < kStages; ++c) mbar_wait(b_full + 8 * c, par, &never);
+      }
+    }
+    __syncthreads();
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (wid == kEpiWarps + 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
+
+__global__ void csr_to_dense_kernel(int n, int lda, const int* __restrict__ rp,
+                                    const int* __restrict__ ci, const double* __restrict__ v,
+                                    double* __restrict__ A) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    double* row = A + (size_t)i * lda;
+    for (int p = rp[i]; p < rp[i + 1]; ++p) row[ci[p]] = v[p];
+  }
+}
+
+// out (n x n) = A with its columns in the order colperm
+__global__ void unscramble_kernel(int n, int lda, const int* __restrict__ colperm,
+                                  const double* __restrict__ A, double* __restrict__ out) {
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)n * n;
+       t += (size_t)gridDim.x * blockDim.x) {
+    const int i = (int)(t / n), c = (int)(t % n);
+    out[t] = A[(size_t)i * lda + colperm[c]];
+  }
+}
+
+// The sub-panels of one step: LU of the m x kb panel copy X.
+template <int W, int R>
+int lu_panel(int m, int kb, int k0, double* X, int* piv, DevFlags* flags, cudaStream_t s) {
+  MSP_CUDA_TRY(cudaFuncSetAttribute(lu_panel_kernel<W, R>,
+                                    cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  for (int c0 = 0; c0 < kb; c0 += W) {
+    const int w = std::min(W, kb - c0), rows = m - c0;
+    // about 128 rows per CTA: more CTAs make the barrier dearer, fewer the rank-1 updates
+    int nct = 1;
+    while (nct < kMaxCluster && nct * 128 < rows) nct *= 2;
+    const int rpc = std::max(W, (rows + nct - 1) / nct);  // CTA 0 holds the rows c0..c0+w-1
+    const int threads = std::max(kP, (int)div_up(div_up(rpc, R), kWarp) * kWarp);
+    if (threads > kLuThreads) return MSP_ERR_ARG;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(nct);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = nct;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    MSP_CUDA_TRY(
+        cudaLaunchKernelEx(&cfg, lu_panel_kernel<W, R>, m, c0, w, kb, rpc, X, piv, k0, flags));
+    MSP_TRY(launch_status());
+    if (c0 + w < kb && m > c0 + w) {
+      lu_update_kernel<W><<<div_up(m - c0 - w, kUpdRows), 256, 0, s>>>(m, c0, w, kb, X);
+      MSP_TRY(launch_status());
+    }
+  }
+  return MSP_OK;
+}
+
+}  // namespace
+
+int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v, double* out,
+                           DevFlags* flags, cudaStream_t s) {
+  if (n <= 0) return MSP_ERR_ARG;
+  const int lda = (int)(div_up(n, kP) * kP), nrt = (int)div_up(n, kRowTile);
+  const int nct = (int)div_up(n, kColTile);
+  const size_t rows = (size_t)nrt * kRowTile;
+  DevBuf<double> A, X, Y, D;
+  DevBuf<char> SA, ST, SD;
+  DevBuf<int> ea, et, ed, piv, pivots, perm, cols_d;
+  MSP_TRY(A.alloc(rows * lda));
+  MSP_TRY(X.alloc((size_t)n * kP));
+  MSP_TRY(Y.alloc(rows * kP));
+  MSP_TRY(D.alloc(kP * kP));
+  MSP_TRY(SA.alloc((size_t)nrt * kTileA));
+  MSP_TRY(ST.alloc((size_t)(lda / kColTile) * kTileB));
+  MSP_TRY(SD.alloc((size_t)kKTiles * kTileB));
+  MSP_TRY(ea.alloc(rows));
+  MSP_TRY(et.alloc(lda));
+  MSP_TRY(ed.alloc(kP));
+  MSP_TRY(piv.alloc(kP));
+  MSP_TRY(pivots.alloc((size_t)lda));
+  MSP_TRY(perm.alloc(1 + 4 * kP));
+  MSP_TRY(cols_d.alloc(n));
+  MSP_CUDA_TRY(cudaMemsetAsync(A.p, 0, rows * lda * sizeof(double), s));
+  csr_to_dense_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, lda, rp, ci, v, A.p);
+  MSP_TRY(launch_status());
+  const size_t diag_smem = sizeof(double) * (kP * (kP + 1) + kP);
+  MSP_CUDA_TRY(cudaFuncSetAttribute(diag_inverse_panel_kernel,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem));
+  for (auto* k : {slice_gemm_kernel<kUpdate>, slice_gemm_kernel<kFirst>, slice_gemm_kernel<kResid>,
+                  slice_gemm_kernel<kCorrect>})
+    MSP_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kGemmSmem));
+  const size_t swap_smem = sizeof(double) * 2 * kP * (kColTile + 1);
+  MSP_CUDA_TRY(cudaFuncSetAttribute(swap_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)swap_smem));
+  const unsigned srow = div_up(rows, 32);
+  for (int k0 = 0; k0 < n; k0 += kP) {
+    const int kb = std::min(kP, n - k0), m = n - k0;
+    panel_copy_kernel<<<grid_for((size_t)m * kP, 256), 256, 0, s>>>(m, k0, kb, lda, A.p, X.p);
+    MSP_TRY(launch_status());
+    // the widest sub-panel whose rows fit the registers of one cluster
+    constexpr int kLuRows = kMaxCluster * kLuThreads;
+    if (m <= kLuRows)
+      MSP_TRY((lu_panel<16, 1>(m, kb, k0, X.p, piv.p, flags, s)));
+    else if (m <= 2 * kLuRows)
+      MSP_TRY((lu_panel<8, 2>(m, kb, k0, X.p, piv.p, flags, s)));
+    else if (m <= 4 * kLuRows)
+      MSP_TRY((lu_panel<4, 4>(m, kb, k0, X.p, piv.p, flags, s)));
+    else if (m <= 16 * kLuRows)
+      MSP_TRY((lu_panel<2, 16>(m, kb, k0, X.p, piv.p, flags, s)));
+    else
+      return MSP_ERR_NOMEM;  // two dense copies of such a matrix exceed the device
+    diag_inverse_panel_kernel<<<kP / kDiagWarps + 1, kDiagWarps * kWarp, diag_smem, s>>>(
+        k0, kb, X.p, piv.p, D.p, SD.p, ed.p, perm.p, pivots.p);
+    MSP_TRY(launch_status());
+    swap_slice_kernel<<<lda / kColTile, 256, swap_smem, s>>>(lda, k0, kb, A.p, perm.p, ST.p, et.p);
+    MSP_TRY(launch_status());
+    // P = -A_iK D (D for the rows K), then one correction: with the digit products the
+    // residual P A_KK + A_iK is nearly exact, so P ends as accurate as its last rounding,
+    // however the explicit inverse D of an ill-conditioned block was
+    const unsigned pt = (unsigned)std::min(sm_count(), nrt * kKTiles);
+    double* AK = A.p + k0;
+    const char* SK = ST.p + (size_t)(k0 / kColTile) * kTileB;
+    slice_rows_kernel<<<srow, 256, 0, s>>>(lda, k0, k0, k0 + kb, A.p, SA.p, ea.p, Y.p);
+    MSP_TRY(launch_status());
+    slice_gemm_kernel<kFirst><<<pt, kGemmThreads, kGemmSmem, s>>>(
+        lda, k0, kb, nrt, kKTiles, 0, AK, SA.p, ea.p, SD.p, ed.p, D.p, flags);
+    MSP_TRY(launch_status());
+    slice_rows_kernel<<<srow, 256, 0, s>>>(lda, k0, 0, 0, A.p, SA.p, ea.p, nullptr);
+    MSP_TRY(launch_status());
+    slice_gemm_kernel<kResid><<<pt, kGemmThreads, kGemmSmem, s>>>(
+        kP, k0, kb, nrt, kKTiles, 0, Y.p, SA.p, ea.p, SK, et.p + k0, D.p, flags);
+    MSP_TRY(launch_status());
+    slice_rows_kernel<<<srow, 256, 0, s>>>(kP, 0, 0, 0, Y.p, SA.p, ea.p, nullptr);
+    MSP_TRY(launch_status());
+    slice_gemm_kernel<kCorrect><<<pt, kGemmThreads, kGemmSmem, s>>>(
+        lda, k0, kb, nrt, kKTiles, 0, AK, SA.p, ea.p, SD.p, ed.p, D.p, flags);
+    MSP_TRY(launch_status());
+    const int ncu = nct - std::min(nct - k0 / kColTile, kKTiles);
+    if (ncu <= 0) continue;
+    slice_rows_kernel<<<srow, 256, 0, s>>>(lda, k0, 0, 0, A.p, SA.p, ea.p, nullptr);
+    MSP_TRY(launch_status());
+    const long long tiles = (long long)nrt * ncu;
+    slice_gemm_kernel<kUpdate><<<(unsigned)std::min<long long>(sm_count(), tiles), kGemmThreads,
+                                 kGemmSmem, s>>>(lda, k0, kb, nrt, ncu, k0 / kColTile, A.p, SA.p,
+                                                 ea.p, ST.p, et.p, D.p, flags);
+    MSP_TRY(launch_status());
+  }
+  std::vector<int> hp(n), cols(n);
+  DevFlags hf{};
+  MSP_CUDA_TRY(cudaMemcpyAsync(hp.data(), pivots.p, n * sizeof(int), cudaMemcpyDeviceToHost, s));
+  MSP_CUDA_TRY(cudaMemcpyAsync(&hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, s));
+  MSP_CUDA_TRY(cudaStreamSynchronize(s));
+  if (hf.code != MSP_OK) return hf.code;
+  for (int c = 0; c < n; ++c) cols[c] = c;
+  for (int k = n - 1; k >= 0; --k)
+    if (hp[k] != k) std::swap(cols[k], cols[hp[k]]);
+  MSP_CUDA_TRY(cudaMemcpyAsync(cols_d.p, cols.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
+  unscramble_kernel<<<grid_for((size_t)n * n, 256), 256, 0, s>>>(n, lda, cols_d.p, A.p, out);
+  MSP_TRY(launch_status());
+  MSP_CUDA_TRY(cudaStreamSynchronize(s));  // cols and the temporaries are in use until here
+  return MSP_OK;
+}
+
+}  // namespace msp

@@ -761,42 +761,11 @@ int level_extras(msp_handle h, Level& L, bool smoothed, bool ell, cudaStream_t s
   return MSP_OK;
 }
 
-// dense inverse of the coarsest matrix by in-place Gauss-Jordan (partial pivoting)
+// dense inverse of the coarsest matrix (coarse_inverse.cu)
 int coarse_inverse(msp_handle h, const DCsr& C, cudaStream_t s) {
   const int n = C.n;
-  DevBuf<double> A, col;
-  DevBuf<int> piv, cp;
-  MSP_TRY(A.alloc((size_t)n * n));
-  MSP_TRY(col.alloc(n));
-  MSP_TRY(piv.alloc(n));
-  MSP_TRY(cp.alloc(n));
   MSP_TRY(h->cinv.alloc((size_t)n * n));
-  MSP_TRY(launch_csr_to_dense(n, C.rp.p, C.ci.p, C.v.p, A.p, s));
-  // blocked: the steps of a panel of 32 columns transform the panel only, then one
-  // rank-32 update applies them to the other columns (row swaps act on whole rows)
-  constexpr int kPanel = 32;
-  DevBuf<double> T;
-  MSP_TRY(T.alloc((size_t)kPanel * n));
-  for (int k0 = 0; k0 < n; k0 += kPanel) {
-    const int nb = std::min(kPanel, n - k0);
-    for (int k = k0; k < k0 + nb; ++k) {
-      MSP_TRY(launch_gj_pivot(n, k, k0, k0 + nb, A.p, col.p, piv.p, h->flags.p, s));
-      MSP_TRY(launch_gj_update(n, k, k0, nb, A.p, col.p, s));
-    }
-    MSP_CUDA_TRY(cudaMemcpyAsync(T.p, A.p + (size_t)k0 * n, (size_t)nb * n * sizeof(double),
-                                 cudaMemcpyDeviceToDevice, s));
-    MSP_TRY(launch_gj_panel_apply(n, k0, nb, A.p, T.p, s));
-  }
-  if (sync_flags(h, s) != MSP_OK) return h->h_flags->code;
-  std::vector<int> hp(n), cols(n);
-  MSP_CUDA_TRY(cudaMemcpyAsync(hp.data(), piv.p, n * sizeof(int), cudaMemcpyDeviceToHost, s));
-  MSP_CUDA_TRY(cudaStreamSynchronize(s));
-  for (int c = 0; c < n; ++c) cols[c] = c;
-  for (int k = n - 1; k >= 0; --k)
-    if (hp[k] != k) std::swap(cols[k], cols[hp[k]]);
-  MSP_CUDA_TRY(cudaMemcpyAsync(cp.p, cols.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
-  MSP_TRY(launch_gj_unscramble(n, cp.p, A.p, h->cinv.p, s));
-  MSP_CUDA_TRY(cudaStreamSynchronize(s));
+  MSP_TRY(coarse_inverse_blocked(n, C.rp.p, C.ci.p, C.v.p, h->cinv.p, h->flags.p, s));
   h->ncoarse = n;
   return MSP_OK;
 }
