@@ -28,6 +28,11 @@ template <typename T>
 int launch_bsr_spmv(int b, int nb, const int* rp, const int* ci, const T* v, const T* x,
                     const T* g, T* y, bool residual, cudaStream_t s,
                     const unsigned char* rmask = nullptr, LongRows lr = LongRows());
+// y[perm[i]] = sum_j A_ij x[perm[j]]: the product in the order perm maps to (x 16-byte
+// aligned, not overlapping y)
+int launch_bsr_spmv_perm(int b, int nb, const int* rp, const int* ci, const double* v,
+                         const int* perm, const double* x, double* y, cudaStream_t s,
+                         LongRows lr);
 // rP[i] = omega_i^T (g_i - (A w)_i)   (omega == nullptr: first unknown only); r != nullptr
 // also receives g - A w
 template <typename T>
@@ -49,12 +54,13 @@ int launch_extract_col0(size_t nnzb, int b, const T* v, T* c0, cudaStream_t s);
 // from zero (later colours still hold zero).
 template <typename T>
 int launch_bgs_colour(int b, int r0, int r1, const int* rp, const int* ci, const int* dpos,
-                      const T* aN, const T* y, T* w, bool lower_only, bool zero_pressure,
-                      cudaStream_t s, const unsigned char* rmask = nullptr,
-                      LongRows lr = LongRows());
-// y[i*(b-1) + r] = (D_N,i^-1 g_i)[r] over the concentration unknowns of every block row
+                      const T* aN, const T* y, T* w, bool lower_only, cudaStream_t s,
+                      const unsigned char* rmask = nullptr, LongRows lr = LongRows());
+// y[i*(b-1) + r] = (D_N,i^-1 g_i)[r] over the concentration unknowns of every block row;
+// w (stride b): pressure slots 0, and y for the rows below rfirst
 template <typename T>
-int launch_nscale(int b, int nb, const T* dNinv, const T* g, T* y, cudaStream_t s);
+int launch_nscale(int b, int nb, const T* dNinv, const T* g, T* y, T* w, int rfirst, cudaStream_t s,
+                  const unsigned char* rmask = nullptr);
 // stage R: forward y_i = r_i - sum_{j<i} L_ij y_j and backward x_i = U_ii^-1 (y_i -
 // sum_{j>i} U_ij x_j); the backward sweep also adds x_i into w.
 template <typename T>
@@ -148,14 +154,16 @@ int launch_reduce_partials(int K, int nblocks, const double* partial, double* ou
 int launch_multi_axpy_norm(size_t n, const double* V, size_t ldv, int K, const double* h,
                            double* w, double* partial, int nblocks, cudaStream_t s,
                            const int* gate = nullptr);
-// v = w / sqrt(nrm2[0]) (nothing when the norm is zero); hn[0] = sqrt(nrm2[0])
-int launch_normalize(size_t n, const double* w, const double* nrm2, double* v, double* hn,
+// v = w / sqrt(nrm2[0]) (nothing when the norm is zero); hn[0] = sqrt(nrm2[0]); c = v in T
+template <typename T>
+int launch_normalize(size_t n, const double* w, const double* nrm2, double* v, double* hn, T* c,
                      cudaStream_t s);
 // x += sum_k y[k] Z[k]
 int launch_update_x(size_t n, const double* Z, size_t ldz, int K, const double* y, double* x,
                     cudaStream_t s);
-// v = r / beta (beta a host scalar)
-int launch_scale(size_t n, const double* r, double alpha, double* v, cudaStream_t s);
+// v = alpha r (alpha a host scalar); c = v in T
+template <typename T>
+int launch_scale(size_t n, const double* r, double alpha, double* v, T* c, cudaStream_t s);
 // partial[blk] = sum of x^2 over the block
 int launch_norm2_partial(size_t n, const double* x, double* partial, int nblocks,
                          cudaStream_t s);

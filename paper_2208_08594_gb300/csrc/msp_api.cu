@@ -1314,21 +1314,22 @@ int stage_N(msp_handle h, const PView<T>& P, const T* g, T* w, cudaStream_t s) {
   {
     Probe pr("stageN_scale", (double)h->nb * (bn * bn + 2 * bn) * sT, s, 1,
              sT == 8 ? 2.0 * (double)h->nb * bn * bn : 0.0);
-    MSP_TRY(launch_nscale<T>(b, h->nb, P.dNinv, g, P.ny, s));
+    MSP_TRY(launch_nscale<T>(b, h->nb, P.dNinv, g, P.ny, w, h->cptr0[1], s, P.m0));
   }
+  // the first colour of the first sweep is done by the scaling
   double bytes = 0.0, fmas = 0.0;
   for (int sw = 0; sw < h->cfg.bgs_sweeps; ++sw)
-    for (int c = 0; c < h->g0; ++c) {
+    for (int c = sw == 0 ? 1 : 0; c < h->g0; ++c) {
       const long long used = h->cc0.lower[c] + (sw == 0 ? 0 : h->cc0.upper[c]);
       bytes += sweep_bytes(h->cptr0[c], h->cptr0[c + 1], used, bn * bn * sT + 4,
                            (2 * bn + 1) * sT + 12);
       fmas += (double)used * bn * bn;
     }
-  Probe pr("stageN_bgs_sweep", bytes, s, h->cfg.bgs_sweeps * h->g0, sT == 8 ? 2.0 * fmas : 0.0);
+  Probe pr("stageN_bgs_sweep", bytes, s, h->cfg.bgs_sweeps * h->g0 - 1, sT == 8 ? 2.0 * fmas : 0.0);
   for (int sw = 0; sw < h->cfg.bgs_sweeps; ++sw)
-    for (int c = 0; c < h->g0; ++c)
+    for (int c = sw == 0 ? 1 : 0; c < h->g0; ++c)
       MSP_TRY(launch_bgs_colour<T>(b, h->cptr0[c], h->cptr0[c + 1], h->rp.p, h->ci.p, h->dpos.p,
-                                   P.aN, P.ny, w, sw == 0, sw == 0, s, P.m0,
+                                   P.aN, P.ny, w, sw == 0, s, P.m0,
                                    long_rows(h, h->cptr0[c], h->cptr0[c + 1])));
   return MSP_OK;
 }
@@ -1521,24 +1522,26 @@ int capture_graph(msp_handle h) {
 
 // w = B g on FP64 colour-ordered vectors, in the configured precision.  Replays the
 // captured graph, except while every launch is timed (stats mode 2).
-int apply_precond_run(msp_handle h, const double* g, double* w, cudaStream_t s);
+int apply_precond_run(msp_handle h, const double* g, double* w, cudaStream_t s, bool staged);
 
 // dot_j >= 0 (the single solve's step j, g = u_j): the application also leaves the dot
 // products u_k . u_j, k <= j, in gs_d[0..j].  The device index is written only when it does
-// not already hold dot_j (in a cycle, only at its first step).
-int apply_precond(msp_handle h, const double* g, double* w, cudaStream_t s, int dot_j = -1) {
+// not already hold dot_j (in a cycle, only at its first step).  staged: g is already in the
+// graph's input buffer too (pg64, or g32 with the FP32 preconditioner).
+int apply_precond(msp_handle h, const double* g, double* w, cudaStream_t s, int dot_j = -1,
+                  bool staged = false) {
   if (dot_j < -1 || dot_j + 1 > kKrylovMaxK) return MSP_ERR_ARG;
   if (h->dot_j_dev != dot_j) {
     h->dot_j_dev = kDotUnknown;
     MSP_TRY(launch_set_int(h->dot_j.p, dot_j, s));
   }
   h->dot_j_dev = kDotUnknown;
-  MSP_TRY(apply_precond_run(h, g, w, s));
+  MSP_TRY(apply_precond_run(h, g, w, s, staged));
   h->dot_j_dev = dot_j >= 0 ? dot_j + 1 : -1;
   return MSP_OK;
 }
 
-int apply_precond_run(msp_handle h, const double* g, double* w, cudaStream_t s) {
+int apply_precond_run(msp_handle h, const double* g, double* w, cudaStream_t s, bool staged) {
   NvtxRange nvtx("msp:precond");
   const size_t n = (size_t)h->nb * h->b;
   const bool fp32 = h->cfg.precision == MSP_PRECISION_FP32;
@@ -1553,10 +1556,11 @@ int apply_precond_run(msp_handle h, const double* g, double* w, cudaStream_t s) 
   // stats mode 3 replays a graph with event nodes around every site; other modes a plain one
   if (h->graph && h->graph_timed != (g_stats_mode == 3)) drop_graph(h);
   if (!h->graph) MSP_TRY(capture_graph(h));
-  if (fp32)
-    MSP_TRY(launch_cast_d2f(n, g, h->g32.p, s));
-  else
+  if (fp32) {
+    if (!staged) MSP_TRY(launch_cast_d2f(n, g, h->g32.p, s));
+  } else if (!staged && g != h->pg64.p) {
     MSP_CUDA_TRY(cudaMemcpyAsync(h->pg64.p, g, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  }
   if (h->graph_timed) {  // this replay re-records the events of the previous one
     std::lock_guard<std::mutex> lk(g_stats_mu);
     resolve_pending();
@@ -1576,6 +1580,7 @@ int apply_precond_run(msp_handle h, const double* g, double* w, cudaStream_t s) 
     }
   }
   if (fp32) return launch_cast_f2d(n, h->w32.p, w, s);
+  if (w == h->pw64.p) return MSP_OK;
   MSP_CUDA_TRY(cudaMemcpyAsync(w, h->pw64.p, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
   return MSP_OK;
 }
@@ -1682,7 +1687,10 @@ int fgmres(msp_handle h, double tol, int* iters, double* relres, double* relres_
       break;
     }
     if (it >= h->cfg.max_it) break;
-    MSP_TRY(launch_scale(n, h->rvec.p, 1.0 / beta, V, s));
+    // the basis vectors also go to the preconditioner's input buffer as they are made
+    const bool fp32 = h->cfg.precision == MSP_PRECISION_FP32;
+    MSP_TRY(fp32 ? launch_scale<float>(n, h->rvec.p, 1.0 / beta, V, h->g32.p, s)
+                 : launch_scale<double>(n, h->rvec.p, 1.0 / beta, V, h->pg64.p, s));
     std::fill(sv.begin(), sv.end(), 0.0);
     int j_used = 0;
     bool breakdown = false;
@@ -1755,7 +1763,7 @@ int fgmres(msp_handle h, double tol, int* iters, double* relres, double* relres_
       double* vj = V + (size_t)j * n;
       double* zj = Z + (size_t)j * n;
       double* w = V + (size_t)(j + 1) * n;
-      MSP_TRY(apply_precond(h, vj, zj, s, j));  // also gs_d[0..j] = u_k . u_j
+      MSP_TRY(apply_precond(h, vj, zj, s, j, true));  // also gs_d[0..j] = u_k . u_j
       stats_add_bytes("krylov_basis_dot", (j + 2.0) * n * 8.0, 2.0 * (j + 1) * n);
       {
         Probe pr("krylov_spmv", bsr_bytes(h, 8.0, 1), s, 1, 2.0 * bsr_fmas(h));
@@ -1777,7 +1785,8 @@ int fgmres(msp_handle h, double tol, int* iters, double* relres, double* relres_
         MSP_TRY(launch_multi_axpy_norm(n, V, n, j + 1, h->gs_g.p, w, h->partial.p, nbk, s));
       }
       MSP_TRY(launch_reduce_partials(1, nbk, h->partial.p, h->nrm.p, false, s));
-      MSP_TRY(launch_normalize(n, w, h->nrm.p, w, h->nrm.p + 1, s));
+      MSP_TRY(fp32 ? launch_normalize<float>(n, w, h->nrm.p, w, h->nrm.p + 1, h->g32.p, s)
+                   : launch_normalize<double>(n, w, h->nrm.p, w, h->nrm.p + 1, h->pg64.p, s));
       MSP_TRY(fetch_out());
       const double hn = hp[150];
       if (!std::isfinite(hn) || !std::isfinite(hp[145])) return MSP_ERR_NONFINITE;
@@ -2561,9 +2570,10 @@ int msp_apply_precond(msp_handle h, const double* d_g, double* d_w, void* stream
   cudaStream_t s = (cudaStream_t)stream;
   if (h->batch) MSP_CUDA_TRY(cudaMemsetAsync(h->rmask0.p, 1, h->nb, s));  // every row
   try {
-    MSP_TRY(launch_gather_blocks(h->nb, h->b, h->perm0.p, d_g, h->bperm.p, s));
-    MSP_TRY(apply_precond(h, h->bperm.p, h->xperm.p, s));
-    MSP_TRY(launch_scatter_blocks(h->nb, h->b, h->perm0.p, h->xperm.p, d_w, s));
+    // straight into and out of the graph's buffers
+    MSP_TRY(launch_gather_blocks(h->nb, h->b, h->perm0.p, d_g, h->pg64.p, s));
+    MSP_TRY(apply_precond(h, h->pg64.p, h->pw64.p, s));
+    MSP_TRY(launch_scatter_blocks(h->nb, h->b, h->perm0.p, h->pw64.p, d_w, s));
     MSP_CUDA_TRY(cudaStreamSynchronize(s));
     return MSP_OK;
   } catch (...) {
@@ -2574,14 +2584,24 @@ int msp_apply_precond(msp_handle h, const double* d_g, double* d_w, void* stream
 int msp_spmv(msp_handle h, const double* d_x, double* d_y, void* stream) {
   if (!h || !d_x || !d_y) return MSP_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  MSP_TRY(launch_gather_blocks(h->nb, h->b, h->perm0.p, d_x, h->bperm.p, s));
-  {
+  const size_t n = (size_t)h->nb * h->b;
+  // straight on the caller's vectors where the vector loads may be used on x and no row of y
+  // is written while x is read; otherwise through colour-ordered copies
+  const bool direct = reinterpret_cast<uintptr_t>(d_x) % 16 == 0 && (d_y + n <= d_x || d_x + n <= d_y);
+  if (direct) {
     Probe pr("api_spmv", bsr_bytes(h, 8.0, 1), s);
-    MSP_TRY(launch_bsr_spmv<double>(h->b, h->nb, h->rp.p, h->ci.p, h->vals.p, h->bperm.p,
-                                    nullptr, h->xperm.p, false, s, nullptr,
-                                    long_rows(h, 0, h->nb)));
+    MSP_TRY(launch_bsr_spmv_perm(h->b, h->nb, h->rp.p, h->ci.p, h->vals.p, h->perm0.p, d_x, d_y, s,
+                                 long_rows(h, 0, h->nb)));
+  } else {
+    MSP_TRY(launch_gather_blocks(h->nb, h->b, h->perm0.p, d_x, h->bperm.p, s));
+    {
+      Probe pr("api_spmv", bsr_bytes(h, 8.0, 1), s);
+      MSP_TRY(launch_bsr_spmv<double>(h->b, h->nb, h->rp.p, h->ci.p, h->vals.p, h->bperm.p,
+                                      nullptr, h->xperm.p, false, s, nullptr,
+                                      long_rows(h, 0, h->nb)));
+    }
+    MSP_TRY(launch_scatter_blocks(h->nb, h->b, h->perm0.p, h->xperm.p, d_y, s));
   }
-  MSP_TRY(launch_scatter_blocks(h->nb, h->b, h->perm0.p, h->xperm.p, d_y, s));
   MSP_CUDA_TRY(cudaStreamSynchronize(s));
   return MSP_OK;
 }

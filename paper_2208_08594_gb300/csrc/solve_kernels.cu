@@ -102,7 +102,7 @@ __device__ __forceinline__ T group_sum(T v) {
 template <int R, int C, typename T>
 __device__ __forceinline__ T block_row_sum(int q0, int q1, int skip, const int* __restrict__ ci,
                                            const T* __restrict__ vals, const T* x, int xs,
-                                           int xo) {
+                                           int xo, const int* __restrict__ perm = nullptr) {
   constexpr int NB = kThreads / R, G = 8;
   __shared__ T part_s[kThreads];
   __shared__ T group_s[G * 8];
@@ -113,7 +113,8 @@ __device__ __forceinline__ T block_row_sum(int q0, int q1, int skip, const int* 
 #pragma unroll 1
     for (int q = q0 + k0; q < q1; q += NB) {
       if (q == skip) continue;
-      const T* xr = x + (size_t)__ldg(ci + q) * xs + xo;
+      const int j = __ldg(ci + q);
+      const T* xr = x + (size_t)(perm ? __ldg(perm + j) : j) * xs + xo;
       const T* a = vals + ((size_t)q * R + r) * C;
 #pragma unroll
       for (int c = 0; c < C; ++c) part = fma(__ldg(a + c), __ldg(xr + c), part);
@@ -205,18 +206,19 @@ template <int B, typename T, bool PDL>
 __global__ void __launch_bounds__(kThreads) bgs_long_colour_kernel(
     int r0, const int* __restrict__ rp, const int* __restrict__ ci, const int* __restrict__ dpos,
     const T* __restrict__ aN, const T* __restrict__ y, T* __restrict__ w, bool lower_only,
-    bool zero_pressure, const unsigned char* __restrict__ rmask) {
+    const unsigned char* __restrict__ rmask) {
   constexpr int BN = B - 1;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int i = r0 + blockIdx.x;
-  if (rmask && !rmask[i]) return;  // uniform over the block
+  if (rmask && !rmask[i]) {  // uniform over the block; later launches rely on the wait
+    if constexpr (PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   const int pd = __ldg(dpos + i);
   const int l = threadIdx.x;
-  const T yl = l < BN ? __ldg(y + (size_t)i * BN + l) : T(0);
   const T sl = long_colour_row_sum<BN, BN, T, PDL>(__ldg(rp + i), lower_only ? pd : __ldg(rp + i + 1),
                                                    pd, ci, aN, w, B, 1);
-  if (l < BN) w[(size_t)i * B + 1 + l] = yl - sl;
-  if (zero_pressure && l == 0) w[(size_t)i * B] = T(0);
+  if (l < BN) w[(size_t)i * B + 1 + l] = __ldcg(y + (size_t)i * BN + l) - sl;
 }
 
 // BILU(0) forward over a colour of long rows only
@@ -227,7 +229,10 @@ __global__ void __launch_bounds__(kThreads) bilu_fwd_long_colour_kernel(
     const unsigned char* __restrict__ rmask) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int i = r0 + blockIdx.x;
-  if (rmask && !rmask[i]) return;
+  if (rmask && !rmask[i]) {  // as in the stage-N sweep
+    if constexpr (PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   const int l = threadIdx.x;
   const T rl = l < B ? __ldg(r + (size_t)i * B + l) : T(0);
   const T sl = long_colour_row_sum<B, B, T, PDL>(__ldg(rp + i), __ldg(dpos + i), -1, ci, lu, y, B, 0);
@@ -242,7 +247,10 @@ __global__ void __launch_bounds__(kThreads) bilu_bwd_long_colour_kernel(
     T* __restrict__ x, T* __restrict__ w, const unsigned char* __restrict__ rmask) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int i = r0 + blockIdx.x;
-  if (rmask && !rmask[i]) return;
+  if (rmask && !rmask[i]) {  // as in the stage-N sweep
+    if constexpr (PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   const int l = threadIdx.x;
   const T sl = long_colour_row_sum<B, B, T, PDL>(__ldg(dpos + i) + 1, __ldg(rp + i + 1), -1, ci, lu,
                                                  x, B, 0);
@@ -268,8 +276,11 @@ inline unsigned with_long_rows(unsigned grid, int nlong) {
 
 // ----------------------------------------------------------------------------------
 // y = A x  or  y = g - A x
+// PERM: x and y in the caller's order (row i of the colour order is row perm[i] of theirs):
+// one launch instead of a gather, the product and a scatter, for one more trip to the
+// permutation per block (132k rows, b = 4, with the call: 58 -> 47 us).
 // ----------------------------------------------------------------------------------
-template <int B, typename T, bool RES>
+template <int B, typename T, bool RES, bool PERM>
 __global__ void __launch_bounds__(kThreads) bsr_spmv_kernel(int nb, const int* __restrict__ rp,
                                                            const int* __restrict__ ci,
                                                            const T* __restrict__ v,
@@ -278,14 +289,17 @@ __global__ void __launch_bounds__(kThreads) bsr_spmv_kernel(int nb, const int* _
                                                            T* __restrict__ y,
                                                            const unsigned char* __restrict__ rmask,
                                                            const int* __restrict__ lrows,
-                                                           int nlong, int lthr) {
+                                                           int nlong, int lthr,
+                                                           const int* __restrict__ perm) {
+  auto at = [&](int j) { return PERM ? __ldg(perm + j) : j; };
   for (int q = blockIdx.x; q < nlong; q += gridDim.x) {  // long rows: a block each
     const int i = lrows[q];
     if (rmask && !rmask[i]) continue;
-    const T sl = block_row_sum<B, B>(__ldg(rp + i), __ldg(rp + i + 1), -1, ci, v, x, B, 0);
+    const T sl = block_row_sum<B, B>(__ldg(rp + i), __ldg(rp + i + 1), -1, ci, v, x, B, 0,
+                                     PERM ? perm : nullptr);
     if (threadIdx.x >= kWarp) continue;  // the row's outputs are warp 0's
     const int l = threadIdx.x;
-    if (l < B) y[(size_t)i * B + l] = RES ? g[(size_t)i * B + l] - sl : sl;
+    if (l < B) y[(size_t)at(i) * B + l] = RES ? g[(size_t)i * B + l] - sl : sl;
   }
   constexpr int GP = Gp<B>::v;
   const int lane = threadIdx.x % GP;
@@ -302,8 +316,8 @@ __global__ void __launch_bounds__(kThreads) bsr_spmv_kernel(int nb, const int* _
       T a0[B], a1[B], x0[B], x1[B];
       load_row<B>(v + ((size_t)p * B + lane) * B, a0);
       load_row<B>(v + ((size_t)(p + 1) * B + lane) * B, a1);
-      load_row<B>(x + (size_t)j0 * B, x0);
-      load_row<B>(x + (size_t)j1 * B, x1);
+      load_row<B>(x + (size_t)at(j0) * B, x0);
+      load_row<B>(x + (size_t)at(j1) * B, x1);
       acc = RES ? fnma_row<B>(a0, x0, acc) : fma_row<B>(a0, x0, acc);
       acc = RES ? fnma_row<B>(a1, x1, acc) : fma_row<B>(a1, x1, acc);
     }
@@ -311,10 +325,10 @@ __global__ void __launch_bounds__(kThreads) bsr_spmv_kernel(int nb, const int* _
       const int j0 = __ldg(ci + p);
       T a0[B], x0[B];
       load_row<B>(v + ((size_t)p * B + lane) * B, a0);
-      load_row<B>(x + (size_t)j0 * B, x0);
+      load_row<B>(x + (size_t)at(j0) * B, x0);
       acc = RES ? fnma_row<B>(a0, x0, acc) : fma_row<B>(a0, x0, acc);
     }
-    y[(size_t)i * B + lane] = acc;
+    y[(size_t)at(i) * B + lane] = acc;
   }
 }
 
@@ -445,92 +459,124 @@ __global__ void extract_col0_kernel(size_t nnzb, int b, const T* __restrict__ v,
 
 // ----------------------------------------------------------------------------------
 // stage N block GS sweep over one colour (BN = b - 1 concentration unknowns)
+// PDL: launched as a programmatic dependent of the previous launch; a row's pointers and
+// the columns and values of its first two blocks are loaded before it waits (w and y are
+// written by earlier launches, so they are read after).
 // ----------------------------------------------------------------------------------
-template <int B, typename T>
+template <int B, typename T, bool PDL>
 __global__ void __launch_bounds__(kThreads) bgs_colour_kernel(
     int r0, int r1, const int* __restrict__ rp, const int* __restrict__ ci,
     const int* __restrict__ dpos, const T* __restrict__ aN, const T* __restrict__ y,
-    T* __restrict__ w, bool lower_only, bool zero_pressure,
-    const unsigned char* __restrict__ rmask, const int* __restrict__ lrows, int nlong,
-    int lthr) {
+    T* w, bool lower_only, const unsigned char* __restrict__ rmask,
+    const int* __restrict__ lrows, int nlong, int lthr) {
   constexpr int BN = B - 1;
   // a colour of long rows may follow as a programmatic dependent (it waits for this grid
   // before it reads w)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  for (int q = blockIdx.x; q < nlong; q += gridDim.x) {  // long rows: a block each
-    const int i = lrows[q];
-    if (rmask && !rmask[i]) continue;
-    const int pd = __ldg(dpos + i);
-    const T sl = block_row_sum<BN, BN>(__ldg(rp + i), lower_only ? pd : __ldg(rp + i + 1), pd,
-                                      ci, aN, w, B, 1);
-    if (threadIdx.x >= kWarp) continue;  // the row's outputs are warp 0's
-    const int l = threadIdx.x;
-    if (l < BN) w[(size_t)i * B + 1 + l] = y[(size_t)i * BN + l] - sl;
-    if (zero_pressure && l == 0) w[(size_t)i * B] = T(0);
+  if ((int)blockIdx.x < nlong) {  // long rows: a block each
+    if constexpr (PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int q = blockIdx.x; q < nlong; q += gridDim.x) {
+      const int i = lrows[q];
+      if (rmask && !rmask[i]) continue;
+      const int pd = __ldg(dpos + i);
+      const T sl = block_row_sum<BN, BN>(__ldg(rp + i), lower_only ? pd : __ldg(rp + i + 1), pd,
+                                        ci, aN, w, B, 1);
+      if (threadIdx.x >= kWarp) continue;  // the row's outputs are warp 0's
+      const int l = threadIdx.x;
+      if (l < BN) w[(size_t)i * B + 1 + l] = __ldcg(y + (size_t)i * BN + l) - sl;
+    }
   }
   // BN consecutive threads per row (thread t: row r0 + t / BN, sub-block row t % BN); a
   // row may straddle two warps, so every lane is busy whatever b is
-  const size_t total = (size_t)(r1 - r0) * BN;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
-       t += (size_t)gridDim.x * blockDim.x) {
-    const int i = r0 + (int)(t / BN), lane = (int)(t % BN);
-    if (rmask && !rmask[i]) continue;
-    T acc = y[(size_t)i * BN + lane];
-    const int p0 = __ldg(rp + i), pd = __ldg(dpos + i), p1 = __ldg(rp + i + 1);
-    if (p1 - p0 > lthr) continue;  // taken by a block above
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const bool in = t < (size_t)(r1 - r0) * BN;
+  const int i = r0 + (int)(t / BN), lane = (int)(t % BN);
+  int p0 = 0, pd = 0, cnt = 0;
+  bool live = in && (!rmask || rmask[i]);
+  if (live) {
+    p0 = __ldg(rp + i);
+    pd = __ldg(dpos + i);
+    const int p1 = __ldg(rp + i + 1);
+    live = p1 - p0 <= lthr;  // else taken by a block above
     const int pend = lower_only ? pd : p1;
     // the off-diagonal blocks only (the diagonal block is not read): the k-th of them
     // sits at p0 + k, one further on from the diagonal position
-    const int cnt = (pend - p0) - (pd < pend ? 1 : 0);
-    auto at = [&](int k) { return p0 + k + (p0 + k >= pd ? 1 : 0); };
-    // w rows of other colours: none of them is written by this launch
-    auto load = [&](int p, T (&a)[BN], T (&xx)[BN]) {
-      const T* xr = w + (size_t)__ldg(ci + p) * B + 1;
-      const T* ar = aN + ((size_t)p * BN + lane) * BN;
-#pragma unroll
-      for (int c = 0; c < BN; ++c) {
-        a[c] = __ldg(ar + c);
-        xx[c] = __ldg(xr + c);
-      }
-    };
-    int k = 0;
-    for (; k + 1 < cnt; k += 2) {  // two blocks in flight, same order as one at a time
-      T a0[BN], x0[BN], a1[BN], x1[BN];
-      load(at(k), a0, x0);
-      load(at(k + 1), a1, x1);
-#pragma unroll
-      for (int c = 0; c < BN; ++c) acc = fma(-a0[c], x0[c], acc);
-#pragma unroll
-      for (int c = 0; c < BN; ++c) acc = fma(-a1[c], x1[c], acc);
-    }
-    if (k < cnt) {
-      T a0[BN], x0[BN];
-      load(at(k), a0, x0);
-#pragma unroll
-      for (int c = 0; c < BN; ++c) acc = fma(-a0[c], x0[c], acc);
-    }
-    // the blocks are D_N,i^-1 A_ij and y_i = D_N,i^-1 g_i: acc is x_i itself
-    w[(size_t)i * B + 1 + lane] = acc;
-    if (zero_pressure && lane == 0) w[(size_t)i * B] = T(0);
+    cnt = (pend - p0) - (pd < pend ? 1 : 0);
   }
+  auto at = [&](int k) { return p0 + k + (p0 + k >= pd ? 1 : 0); };
+  auto load_a = [&](int p, T (&a)[BN]) {
+    const T* ar = aN + ((size_t)p * BN + lane) * BN;
+#pragma unroll
+    for (int c = 0; c < BN; ++c) a[c] = __ldg(ar + c);
+  };
+  // w rows of other colours: none of them is written by this launch
+  auto load_x = [&](int j, T (&xx)[BN]) {
+    const T* xr = w + (size_t)j * B + 1;
+#pragma unroll
+    for (int c = 0; c < BN; ++c) xx[c] = PDL ? xr[c] : __ldg(xr + c);
+  };
+  T a0[BN], a1[BN];
+  int j0 = 0, j1 = 0;
+  if (PDL && live && cnt > 1) {
+    j0 = __ldg(ci + at(0));
+    j1 = __ldg(ci + at(1));
+    load_a(at(0), a0);
+    load_a(at(1), a1);
+  }
+  if constexpr (PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!live) return;
+  T acc = PDL ? __ldcg(y + (size_t)i * BN + lane) : __ldg(y + (size_t)i * BN + lane);
+  int k = 0;
+  for (; k + 1 < cnt; k += 2) {  // two blocks in flight, same order as one at a time
+    if (!PDL || k > 0) {
+      j0 = __ldg(ci + at(k));
+      j1 = __ldg(ci + at(k + 1));
+      load_a(at(k), a0);
+      load_a(at(k + 1), a1);
+    }
+    T x0[BN], x1[BN];
+    load_x(j0, x0);
+    load_x(j1, x1);
+#pragma unroll
+    for (int c = 0; c < BN; ++c) acc = fma(-a0[c], x0[c], acc);
+#pragma unroll
+    for (int c = 0; c < BN; ++c) acc = fma(-a1[c], x1[c], acc);
+  }
+  if (k < cnt) {
+    T x0[BN];
+    load_a(at(k), a0);
+    load_x(__ldg(ci + at(k)), x0);
+#pragma unroll
+    for (int c = 0; c < BN; ++c) acc = fma(-a0[c], x0[c], acc);
+  }
+  // the blocks are D_N,i^-1 A_ij and y_i = D_N,i^-1 g_i: acc is x_i itself
+  w[(size_t)i * B + 1 + lane] = acc;
 }
 
 // y_i = D_N,i^-1 g_i (concentration part of g), once per stage-N application: the sweeps
-// then start every row from y_i and use the pre-scaled blocks
+// then start every row from y_i and use the pre-scaled blocks.  w: pressure slots 0, and for
+// the rows below rfirst (the first colour, which has no earlier colour to read in the sweep
+// from zero) that sweep's result, y_i itself.
 template <int BN, typename T>
 __global__ void nscale_kernel(int nb, const T* __restrict__ dNinv, const T* __restrict__ g,
-                              T* __restrict__ y) {
+                              T* __restrict__ y, T* __restrict__ w, int rfirst,
+                              const unsigned char* __restrict__ rmask) {
   constexpr int B = BN + 1;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const size_t total = (size_t)nb * BN;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
        t += (size_t)gridDim.x * blockDim.x) {
     const size_t i = t / BN;  // row i, concentration unknown t % BN
+    const int c0 = (int)(t % BN);
     const T* d = dNinv + t * BN;
     const T* gi = g + i * B + 1;
     T acc = T(0);
 #pragma unroll
     for (int c = 0; c < BN; ++c) acc = fma(__ldg(d + c), gi[c], acc);
     y[t] = acc;
+    if (rmask && !rmask[i]) continue;
+    if (c0 == 0) w[i * B] = T(0);
+    if (i < (size_t)rfirst) w[i * B + 1 + c0] = acc;
   }
 }
 
@@ -1317,19 +1363,22 @@ __global__ void __launch_bounds__(kThreads) norm2_partial_kernel(size_t n, const
 }
 
 // in place allowed (v == w); multiplies by the reciprocal (an FP64 division per element
-// would make this kernel FP64-ALU bound)
+// would make this kernel FP64-ALU bound).  c: a second copy of v (the preconditioner's
+// input buffer, in its type), so that the next application needs no copy of its own.
+template <typename T>
 __global__ void normalize_kernel(size_t n, const double* w, const double* __restrict__ nrm2,
-                                 double* v, double* __restrict__ hn) {
+                                 double* v, double* __restrict__ hn, T* __restrict__ c) {
   const double h = sqrt(nrm2[0]);
   if (blockIdx.x == 0 && threadIdx.x == 0) hn[0] = h;
   if (h == 0.0) return;
   const double rh = 1.0 / h;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    v[i] = w[i] * rh;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const double x = w[i] * rh;
+    v[i] = x;
+    c[i] = (T)x;
+  }
 }
-
-// DGKS test after one Gram-Schmidt pass: gate = 1 iff ||w_after||^2 < ||w_before||^2 / 2
 
 __global__ void update_x_kernel(size_t n, const double* __restrict__ Z, size_t ldz, int K,
                                 const double* __restrict__ y, double* __restrict__ x) {
@@ -1344,11 +1393,15 @@ __global__ void update_x_kernel(size_t n, const double* __restrict__ Z, size_t l
   }
 }
 
+template <typename T>
 __global__ void scale_kernel(size_t n, const double* __restrict__ r, double alpha,
-                             double* __restrict__ v) {
+                             double* __restrict__ v, T* __restrict__ c) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    v[i] = r[i] * alpha;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const double x = r[i] * alpha;
+    v[i] = x;
+    c[i] = (T)x;
+  }
 }
 
 // ---- batched Krylov: the vector of a block-diagonal system is split into chunks that each
@@ -1635,11 +1688,23 @@ int launch_bsr_spmv(int b, int nb, const int* rp, const int* ci, const T* v, con
   MSP_B_SWITCH(b, {
     const unsigned grid = with_long_rows(grid_groups(nb, Gp<B_>::v), lr.n);
     if (residual)
-      bsr_spmv_kernel<B_, T, true><<<grid, kThreads, 0, s>>>(nb, rp, ci, v, x, g, y, rmask,
-                                                             lr.rows, lr.n, lr.thr);
+      bsr_spmv_kernel<B_, T, true, false><<<grid, kThreads, 0, s>>>(
+          nb, rp, ci, v, x, g, y, rmask, lr.rows, lr.n, lr.thr, nullptr);
     else
-      bsr_spmv_kernel<B_, T, false><<<grid, kThreads, 0, s>>>(nb, rp, ci, v, x, g, y, rmask,
-                                                              lr.rows, lr.n, lr.thr);
+      bsr_spmv_kernel<B_, T, false, false><<<grid, kThreads, 0, s>>>(
+          nb, rp, ci, v, x, g, y, rmask, lr.rows, lr.n, lr.thr, nullptr);
+  });
+  return launch_status();
+}
+
+int launch_bsr_spmv_perm(int b, int nb, const int* rp, const int* ci, const double* v,
+                         const int* perm, const double* x, double* y, cudaStream_t s,
+                         LongRows lr) {
+  if (nb <= 0) return MSP_OK;
+  MSP_B_SWITCH(b, {
+    const unsigned grid = with_long_rows(grid_groups(nb, Gp<B_>::v), lr.n);
+    bsr_spmv_kernel<B_, double, false, true><<<grid, kThreads, 0, s>>>(
+        nb, rp, ci, v, x, nullptr, y, nullptr, lr.rows, lr.n, lr.thr, perm);
   });
   return launch_status();
 }
@@ -1681,38 +1746,32 @@ int launch_extract_col0(size_t nnzb, int b, const T* v, T* c0, cudaStream_t s) {
   return launch_status();
 }
 
+// Threads of a class up to which its launch is a programmatic dependent of the previous
+// one: classes of a few blocks, whose time is the chain of loads that then overlaps the
+// previous launch.  A class that fills the SMs only holds places with waiting blocks: with a
+// limit of 600k threads the 132k-row application lost 2 % (b = 4, 66k rows a class).
+constexpr size_t kBgsPdlThreads = 8192;
+
 template <typename T>
 int launch_bgs_colour(int b, int r0, int r1, const int* rp, const int* ci, const int* dpos,
-                      const T* aN, const T* y, T* w, bool lower_only, bool zero_pressure,
-                      cudaStream_t s, const unsigned char* rmask, LongRows lr) {
+                      const T* aN, const T* y, T* w, bool lower_only, cudaStream_t s,
+                      const unsigned char* rmask, LongRows lr) {
   if (r1 <= r0 || b < 2) return MSP_OK;
-  if (lr.n > 0 && lr.n == r1 - r0) {  // a colour of long rows only (the well rows)
-    switch (b) {
-#define MSP_BGS_LONG_CASE(BB)                                                                  \
-  case BB:                                                                                     \
-    return launch_programmatic(bgs_long_colour_kernel<BB, T, true>, (unsigned)(r1 - r0), s, r0, \
-                               rp, ci, dpos, aN, y, w, lower_only, zero_pressure, rmask);
-      MSP_BGS_LONG_CASE(2)
-      MSP_BGS_LONG_CASE(3)
-      MSP_BGS_LONG_CASE(4)
-      MSP_BGS_LONG_CASE(5)
-      MSP_BGS_LONG_CASE(6)
-      MSP_BGS_LONG_CASE(7)
-      MSP_BGS_LONG_CASE(8)
-#undef MSP_BGS_LONG_CASE
-      default:
-        return MSP_ERR_ARG;
-    }
-  }
+  const size_t threads = (size_t)(r1 - r0) * (b - 1);
+  const unsigned grid = with_long_rows(div_up(threads, kThreads), lr.n);
   switch (b) {
-#define MSP_BGS_CASE(BB)                                                                   \
-  case BB: {                                                                               \
-    const unsigned grid =                                                                  \
-        with_long_rows(grid_for((size_t)(r1 - r0) * (BB - 1), kThreads, kRowGridPerSm), lr.n); \
-    bgs_colour_kernel<BB, T><<<grid, kThreads, 0, s>>>(                                    \
-        r0, r1, rp, ci, dpos, aN, y, w, lower_only, zero_pressure, rmask, lr.rows, lr.n,    \
-        lr.thr);                                                                           \
-  } break;
+#define MSP_BGS_CASE(BB)                                                                      \
+  case BB:                                                                                    \
+    if (lr.n > 0 && lr.n == r1 - r0) /* a colour of long rows only (the well rows) */         \
+      MSP_TRY(launch_programmatic(bgs_long_colour_kernel<BB, T, true>, (unsigned)lr.n, s, r0, \
+                                  rp, ci, dpos, aN, y, w, lower_only, rmask));                \
+    else if (threads <= kBgsPdlThreads)                                                       \
+      MSP_TRY(launch_programmatic(bgs_colour_kernel<BB, T, true>, grid, s, r0, r1, rp, ci,    \
+                                  dpos, aN, y, w, lower_only, rmask, lr.rows, lr.n, lr.thr)); \
+    else                                                                                      \
+      bgs_colour_kernel<BB, T, false><<<grid, kThreads, 0, s>>>(                              \
+          r0, r1, rp, ci, dpos, aN, y, w, lower_only, rmask, lr.rows, lr.n, lr.thr);          \
+    break;
     MSP_BGS_CASE(2)
     MSP_BGS_CASE(3)
     MSP_BGS_CASE(4)
@@ -1728,17 +1787,18 @@ int launch_bgs_colour(int b, int r0, int r1, const int* rp, const int* ci, const
 }
 
 template <typename T>
-int launch_nscale(int b, int nb, const T* dNinv, const T* g, T* y, cudaStream_t s) {
+int launch_nscale(int b, int nb, const T* dNinv, const T* g, T* y, T* w, int rfirst, cudaStream_t s,
+                  const unsigned char* rmask) {
   if (nb <= 0 || b < 2) return MSP_OK;
   const unsigned grid = grid_for((size_t)nb * (b - 1), kThreads);
   switch (b - 1) {
-    case 1: nscale_kernel<1, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y); break;
-    case 2: nscale_kernel<2, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y); break;
-    case 3: nscale_kernel<3, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y); break;
-    case 4: nscale_kernel<4, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y); break;
-    case 5: nscale_kernel<5, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y); break;
-    case 6: nscale_kernel<6, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y); break;
-    case 7: nscale_kernel<7, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y); break;
+    case 1: nscale_kernel<1, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y, w, rfirst, rmask); break;
+    case 2: nscale_kernel<2, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y, w, rfirst, rmask); break;
+    case 3: nscale_kernel<3, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y, w, rfirst, rmask); break;
+    case 4: nscale_kernel<4, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y, w, rfirst, rmask); break;
+    case 5: nscale_kernel<5, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y, w, rfirst, rmask); break;
+    case 6: nscale_kernel<6, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y, w, rfirst, rmask); break;
+    case 7: nscale_kernel<7, T><<<grid, kThreads, 0, s>>>(nb, dNinv, g, y, w, rfirst, rmask); break;
     default: return MSP_ERR_ARG;
   }
   return launch_status();
@@ -2030,9 +2090,10 @@ int launch_norm2_partial(size_t n, const double* x, double* partial, int nblocks
   return launch_status();
 }
 
-int launch_normalize(size_t n, const double* w, const double* nrm2, double* v, double* hn,
+template <typename T>
+int launch_normalize(size_t n, const double* w, const double* nrm2, double* v, double* hn, T* c,
                      cudaStream_t s) {
-  normalize_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(n, w, nrm2, v, hn);
+  normalize_kernel<T><<<grid_for(n, kThreads), kThreads, 0, s>>>(n, w, nrm2, v, hn, c);
   return launch_status();
 }
 
@@ -2044,8 +2105,9 @@ int launch_update_x(size_t n, const double* Z, size_t ldz, int K, const double* 
   return launch_status();
 }
 
-int launch_scale(size_t n, const double* r, double alpha, double* v, cudaStream_t s) {
-  scale_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(n, r, alpha, v);
+template <typename T>
+int launch_scale(size_t n, const double* r, double alpha, double* v, T* c, cudaStream_t s) {
+  scale_kernel<T><<<grid_for(n, kThreads), kThreads, 0, s>>>(n, r, alpha, v, c);
   return launch_status();
 }
 
@@ -2185,9 +2247,10 @@ int launch_scatter_blocks(int nb, int b, const int* perm, const double* in, doub
                                          LongRows);                                          \
   template int launch_extract_col0<T>(size_t, int, const T*, T*, cudaStream_t);             \
   template int launch_bgs_colour<T>(int, int, int, const int*, const int*, const int*,      \
-                                    const T*, const T*, T*, bool, bool, cudaStream_t,       \
+                                    const T*, const T*, T*, bool, cudaStream_t,             \
                                     const unsigned char*, LongRows);                        \
-  template int launch_nscale<T>(int, int, const T*, const T*, T*, cudaStream_t);            \
+  template int launch_nscale<T>(int, int, const T*, const T*, T*, T*, int, cudaStream_t,    \
+                                const unsigned char*);                                      \
   template int launch_bilu_fwd<T>(int, int, int, const int*, const int*, const int*,        \
                                   const T*, const T*, T*, cudaStream_t, const unsigned char*, \
                                   LongRows);                                                \
@@ -2215,7 +2278,10 @@ int launch_scatter_blocks(int nb, int b, const int* perm, const double* in, doub
                                                T*, int, cudaStream_t, const unsigned char*);                       \
   template int launch_prolong_add<T>(int, const int*, const T*, T*, cudaStream_t,             \
                                      const unsigned char*);          \
-  template int launch_dense_gemv<T>(int, const double*, const T*, T*, cudaStream_t);
+  template int launch_dense_gemv<T>(int, const double*, const T*, T*, cudaStream_t);        \
+  template int launch_normalize<T>(size_t, const double*, const double*, double*, double*,  \
+                                   T*, cudaStream_t);                                       \
+  template int launch_scale<T>(size_t, const double*, double, double*, T*, cudaStream_t);
 MSP_INST(double)
 MSP_INST(float)
 #undef MSP_INST
