@@ -511,9 +511,10 @@ int vertices_grouping_gpu(msp_handle h, int n, const DevBuf<int>& srp, const Dev
   MSP_TRY(colour_r.alloc(n));
   MSP_TRY(colour.alloc(n));
   MSP_CUDA_TRY(cudaMemsetAsync(meta.p, 0, 2 * sizeof(int), s));
-  // two-hop lists of the relabelled graph (the second circle of every vertex as one run),
-  // unless they would pass int offsets or 2 GB: then the colouring gathers the rows itself
+  // the lists of the relabelled graph (neighbours and second circle of every vertex), unless
+  // they would pass int offsets or 2 GB: then the colouring gathers the rows itself
   DevBuf<int> tcnt, tp, tl;
+  DevBuf<int4> lists;
   DevBuf<unsigned long long> ttotal;
   MSP_TRY(tcnt.alloc(n));
   MSP_TRY(ttotal.alloc(1));
@@ -521,18 +522,20 @@ int vertices_grouping_gpu(msp_handle h, int n, const DevBuf<int>& srp, const Dev
   unsigned long long htotal = 0;
   MSP_CUDA_TRY(cudaMemcpyAsync(&htotal, ttotal.p, sizeof(htotal), cudaMemcpyDeviceToHost, s));
   MSP_CUDA_TRY(cudaStreamSynchronize(s));
-  const bool twohop = htotal < (1ull << 31) - 1 && htotal * sizeof(int) <= (2ull << 30);
-  if (twohop) {
-    MSP_TRY(tp.alloc((size_t)n + 1));
+  htotal += (unsigned long long)snnz;
+  const int passes = h->cfg.loop_limit > 0 ? h->cfg.loop_limit : n;
+  if (htotal < (1ull << 31) - 1 && htotal * sizeof(int) <= (2ull << 30) && colouring_batch_ok(n)) {
+    MSP_TRY(tp.alloc((size_t)n));
+    MSP_TRY(lists.alloc((size_t)n));
     MSP_TRY(tl.alloc(std::max<size_t>(1, (size_t)htotal)));
     MSP_TRY(exclusive_scan_int(h->ss, n, tcnt.p, tp.p, s));
-    const int last = (int)htotal;
-    MSP_CUDA_TRY(cudaMemcpyAsync(tp.p + n, &last, sizeof(int), cudaMemcpyHostToDevice, s));
-    MSP_TRY(launch_twohop_fill(n, rrp.p, rci.p, tp.p, tl.p, s));
+    MSP_TRY(launch_twohop_lists(n, rrp.p, rci.p, tp.p, tcnt.p, lists.p, tl.p, s));
+    MSP_TRY(launch_colouring_batch(n, lists.p, tl.p, inV.p, wbar.p, bitmap.p, colour_r.p, meta.p,
+                                   passes, s));
+  } else {
+    MSP_TRY(launch_colouring(n, rrp.p, rci.p, inV.p, wbar.p, bitmap.p, words, colour_r.p, meta.p,
+                             passes, s));
   }
-  MSP_TRY(launch_colouring(n, rrp.p, rci.p, twohop ? tp.p : nullptr, twohop ? tl.p : nullptr,
-                           inV.p, wbar.p, bitmap.p, words, colour_r.p, meta.p,
-                           h->cfg.loop_limit > 0 ? h->cfg.loop_limit : n, s));
   map_kernel<<<grid1(n), kThreads, 0, s>>>(n, colour_r.p, rank.p, colour.p);  // colour[v] = colour_r[rank[v]]
   MSP_TRY(launch_status());
   int hm[2] = {0, 0};

@@ -300,22 +300,266 @@ __global__ void segment_sums_kernel(int nseg, const int* __restrict__ seg_start,
 }
 
 // ----------------------------------------------------------------------------------
-// Sequential VerticesGrouping by one warp on the graph relabelled by priority rank
+// Sequential VerticesGrouping by one thread block on the graph relabelled by priority rank
 // (degree desc, index asc), so that the vertex Algorithm 4.1 picks (the largest degree,
-// the smallest index among equals) is simply the smallest label.  inV is a bitmap of the
-// vertices in V of the current pass (test-and-clear with atomics, so the lanes can remove
-// neighbours concurrently); a vertex leaves V when it is coloured or moved to Wbar, and
-// the Wbar list of a pass is V of the next one.  The frontier hat W is a three-level
-// bitmap, so its first set bit is the next pick.  A vertex that leaves V as a neighbour
-// of W leaves the frontier at the same time (the else branch of Algorithm 4.1 would only
-// move it to Wbar, where it already is); an entry found outside V when popped is still
-// dropped.  With an empty frontier the pick is the
-// smallest label still in V (a cursor that only moves forward).  Both bitmaps live in
-// shared memory when they fit.  The second circle is read from the graph's two-hop lists
-// when they are given (one contiguous run per vertex, loaded together with the
-// neighbours); otherwise it is gathered from the neighbours' rows with every lane issuing
-// its loads back to back (owner rows looked up in shared memory).
+// the smallest index among equals) is simply the smallest label.  V of the current pass and
+// the frontier hat W (always a subset of V: a vertex leaving V leaves the frontier too, where
+// the else branch of Algorithm 4.1 would only move it to Wbar, where it already is) are
+// bitmaps; the Wbar list of a pass is V of the next one.  The frontier has two summary
+// levels above its words, whose bits may be stale (set for an empty word) and are corrected
+// when a search meets them, so that clearing a bit touches one word.  The next pick is the
+// frontier's first bit; with an empty frontier the smallest label still in V (a cursor that
+// only moves forward).
+//
+// Batches: the frontier's first kBatch vertices (of one group of 1024 labels) are candidates
+// together, one warp each.  The warps load their candidate's list (neighbours, then the
+// second circle without repeats) and test it against V and the frontier as they are at the
+// start of the batch; from that come, per candidate, which other candidates it would remove
+// from V and the smallest vertex it would add to the frontier.  The picks of the batch
+// follow in order from these: a candidate that an earlier pick removed is passed over, and
+// the batch ends where a vertex that would join the frontier comes before the next
+// candidate.  That is exactly the picks of one at a time: V and the frontier after them are
+// V without the picks and their neighbours, and what lies in that V of the old frontier and
+// of the picks' second circles.
+//
+// Bound by the chain of barriers, shared-memory updates and trips to L2 of a batch (about
+// 2.2 us; 3.4 to 4.5 picks on coarse levels, nearly every candidate on a 7-point grid).  With
+// one pick at a time and the second circle with its repeats: level 1 of the 60x220x85 grid
+// (346k rows) 485 ms, 41k rows 54 ms, the 1.12M cells themselves 2.4 s; now 221, 25 and
+// 250 ms.  (Eight candidates resolved one after the other by one warp: 372 and 44 ms.)
 // ----------------------------------------------------------------------------------
+constexpr int kBatch = 16;   // candidates (warps)
+constexpr int kRegs = 4;     // list entries per lane kept in registers
+
+template <bool VS, bool FS>
+__global__ void __launch_bounds__(32 * kBatch) colouring_batch_kernel(
+    int n, const int4* __restrict__ meta, const int* __restrict__ list, unsigned* gV, unsigned* gF,
+    int* wbar, int* colour, int* result, int max_passes) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int kNone = 0x7fffffff;
+  extern __shared__ unsigned smem_bits[];
+  __shared__ __align__(16) int cand[kBatch], adj[kBatch], mins[kBatch];
+  __shared__ int before[32];  // frontier vertices before each word of the candidates' group
+  __shared__ int s_nc, s_group, s_nwbar;
+  const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
+  const int n0 = (n + 31) / 32, n1 = (n0 + 31) / 32, n2 = (n1 + 31) / 32;
+  volatile unsigned* l2 = smem_bits;
+  volatile unsigned* l1 = smem_bits + n2;
+  unsigned* V = VS ? smem_bits + n2 + n1 : gV;
+  unsigned* F = FS ? smem_bits + n2 + n1 + (VS ? n0 : 0) : gF;
+  for (int k = threadIdx.x; k < n2; k += 32 * kBatch) l2[k] = 0u;
+  for (int k = threadIdx.x; k < n1; k += 32 * kBatch) l1[k] = 0u;
+  for (int k = threadIdx.x; k < n0; k += 32 * kBatch) {
+    const int rem = n - 32 * k;
+    F[k] = 0u;
+    V[k] = rem >= 32 ? kAll : ((1u << rem) - 1u);
+  }
+  auto v_word = [&](int x) { return *(volatile unsigned*)(V + (x >> 5)); };
+  auto f_word = [&](int x) { return *(volatile unsigned*)(F + (x >> 5)); };
+  int coloured = 0, g = 0;
+  while (coloured < n) {  // uniform over the block
+    ++g;
+    if (g > n || g > max_passes) {  // every pass colours at least one vertex
+      if (threadIdx.x == 0) result[1] = 1;
+      return;
+    }
+    int cursor = 0;
+    if (threadIdx.x == 0) s_nwbar = 0;
+    __syncthreads();
+    // every round of this loop picks at least one vertex
+    for (long long rounds = (long long)n - coloured + 1;; --rounds) {
+      if (rounds < 0) {
+        if (threadIdx.x == 0) result[1] = 1;
+        return;
+      }
+      // ---- candidates
+      if (wid == 0) {
+        int nc = 0, group = -1;
+        while (true) {  // each turn ends the search or clears a summary bit
+          int i2 = -1;
+          for (int base = 0; base < n2 && i2 < 0; base += 32) {
+            const unsigned w = base + lane < n2 ? l2[base + lane] : 0u;
+            const unsigned m = __ballot_sync(kAll, w != 0u);
+            if (m) i2 = base + __ffs(m) - 1;
+          }
+          if (i2 < 0) break;
+          const int i1 = i2 * 32 + __ffs(l2[i2]) - 1;
+          const int wi = i1 * 32 + lane;
+          unsigned w = wi < n0 ? *(volatile unsigned*)(F + wi) : 0u;
+          const unsigned m = __ballot_sync(kAll, w != 0u);
+          __syncwarp();
+          if (lane == 0) {
+            l1[i1] = m;
+            if (m == 0u) l2[i2] = l2[i2] & ~(1u << (i1 & 31));
+          }
+          __syncwarp();
+          if (m == 0u) continue;
+          const int cnt = __popc(w);
+          int pre = cnt;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(kAll, pre, o);
+            if (lane >= o) pre += t;
+          }
+          nc = min(kBatch, __shfl_sync(kAll, pre, 31));
+          group = i1;
+          before[lane] = pre - cnt;
+          for (int k = pre - cnt; w != 0u && k < kBatch; ++k) {
+            cand[k] = wi * 32 + __ffs(w) - 1;
+            w &= w - 1u;
+          }
+          break;
+        }
+        if (nc == 0) {
+          while (cursor < n) {  // V by label
+            const int r = cursor + lane;
+            const unsigned m = __ballot_sync(kAll, r < n && ((v_word(min(r, n - 1)) >> (r & 31)) & 1u));
+            if (m) {
+              cursor += __ffs(m) - 1;
+              nc = 1;
+              break;
+            }
+            cursor += 32;
+          }
+          if (lane == 0 && nc) cand[0] = cursor;
+        }
+        if (lane == 0) {
+          s_nc = nc;
+          s_group = group;
+        }
+      }
+      __syncthreads();
+      const int nc = s_nc, group = s_group;
+      if (nc == 0) break;  // V empty: the pass is over
+      // ---- each candidate's list against V and the frontier at the start of the batch
+      int x[kRegs];
+      unsigned near = 0, far = 0;  // entries in V: neighbours; second circle, not in hat W
+      int st = 0, deg = 0, tot = 0, v = 0;
+      if (wid < nc) {
+        v = cand[wid];
+        const int4 mt = __ldg(meta + v);
+        st = mt.x;
+        deg = mt.y;
+        tot = mt.z;
+        unsigned a = 0;
+        int first = kNone;
+        auto test = [&](int e, int y, int u) {
+          const unsigned vw = v_word(y), fw = f_word(y);
+          if (!((vw >> (y & 31)) & 1u)) return;
+          const bool in_f = (fw >> (y & 31)) & 1u;
+          if (e < deg) {
+            if (u < kRegs) near |= 1u << u;
+            if (in_f && (y >> 10) == group) {
+              const int idx = before[(y >> 5) & 31] + __popc(fw & ((1u << (y & 31)) - 1u));
+              if (idx < nc) a |= 1u << idx;
+            }
+          } else if (!in_f) {
+            if (u < kRegs) far |= 1u << u;
+            first = min(first, y);
+          }
+        };
+#pragma unroll
+        for (int u = 0; u < kRegs; ++u) {
+          const int e = lane + 32 * u;
+          x[u] = e < tot ? __ldg(list + st + e) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kRegs; ++u)
+          if (x[u] >= 0) test(lane + 32 * u, x[u], u);
+        for (int e = lane + 32 * kRegs; e < tot; e += 32) test(e, __ldg(list + st + e), kRegs);
+        a = __reduce_or_sync(kAll, a);
+        first = __reduce_min_sync(kAll, first);
+        if (lane == 0) {
+          adj[wid] = (int)a;
+          mins[wid] = first;
+        }
+      }
+      __syncthreads();
+      // ---- the picks (every thread, the same)
+      unsigned picked = 0, removed = 0;
+      {
+        int newmin = kNone;
+#pragma unroll
+        for (int t = 0; t < kBatch; ++t) {
+          const int c = cand[t], m = mins[t];
+          const unsigned ad = (unsigned)adj[t];
+          if (t >= nc || c > newmin) break;  // a vertex that joins the frontier comes first
+          if ((removed >> t) & 1u) continue;  // leaves V with an earlier pick of the batch
+          picked |= 1u << t;
+          removed |= ad;
+          newmin = min(newmin, m);
+        }
+      }
+      const bool mine = (picked >> wid) & 1u;
+      if (mine) {
+        // W = W u {v};  Wbar = Wbar u (S_v n V), V = V / S_v (and hat W with it)
+        if (lane == 0) {
+          atomicAnd(V + (v >> 5), ~(1u << (v & 31)));
+          atomicAnd(F + (v >> 5), ~(1u << (v & 31)));
+          colour[v] = g;
+        }
+        for (int q = 0; q < deg; q += 32) {
+          const int e = q + lane, u = q / 32;
+          int j = -1;
+          if (u < kRegs) {
+#pragma unroll
+            for (int uu = 0; uu < kRegs; ++uu)
+              if (uu == u && ((near >> uu) & 1u)) j = x[uu];
+          } else if (e < deg) {
+            j = __ldg(list + st + e);
+          }
+          bool take = false;
+          if (j >= 0) {
+            const unsigned bit = 1u << (j & 31);
+            take = (atomicAnd(V + (j >> 5), ~bit) & bit) != 0u;  // once, whoever comes first
+            if (take) atomicAnd(F + (j >> 5), ~bit);
+          }
+          const unsigned m = __ballot_sync(kAll, take);
+          if (m) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_nwbar, __popc(m));
+            at = __shfl_sync(kAll, at, 0);
+            if (take) wbar[at + __popc(m & ((1u << lane) - 1u))] = j;
+          }
+        }
+      }
+      coloured += __popc(picked);
+      __syncthreads();
+      if (mine) {
+        // hat W = hat W u hat S_v: undetermined vertices of the second circle
+        auto join = [&](int y) {
+          if (!((v_word(y) >> (y & 31)) & 1u)) return;
+          atomicOr(F + (y >> 5), 1u << (y & 31));
+          atomicOr((unsigned*)l1 + (y >> 10), 1u << ((y >> 5) & 31));
+          atomicOr((unsigned*)l2 + (y >> 15), 1u << ((y >> 10) & 31));
+          // the next picks come from here: their list's place is then an L1 hit
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(meta + y)));
+        };
+#pragma unroll
+        for (int u = 0; u < kRegs; ++u)
+          if ((far >> u) & 1u) join(x[u]);
+        for (int e = max(deg - deg % 32, 32 * kRegs) + lane; e < tot; e += 32)
+          if (e >= deg) join(__ldg(list + st + e));
+      }
+      __syncthreads();
+    }
+    // Wbar of this pass is V of the next one
+    const int nwbar = s_nwbar;
+    for (int t = threadIdx.x; t < nwbar; t += 32 * kBatch) {
+      const int j = wbar[t];
+      atomicOr(V + (j >> 5), 1u << (j & 31));
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) result[0] = g;
+}
+
+// The same one pick at a time, the second circle gathered from the neighbours' rows (every
+// lane issuing its loads back to back, owner rows looked up in shared memory): for callers
+// without room for lists, graphs whose lists would not fit 32-bit offsets (a vertex joined
+// to most of a large graph) and more labels than the batched kernel keeps summaries of.
+constexpr size_t kColouringSmem = 220 * 1024;
+
 struct Bitmap3 {
   unsigned* l0;
   unsigned* l1;
@@ -379,21 +623,12 @@ __device__ __forceinline__ bool in_v(const unsigned* inV, int v) {
 
 constexpr int kSecondU = 8;  // second-circle entries gathered per lane per round
 
-// Fetch the row pointers and two-hop pointers of vertex x into L1 without waiting: the
-// next picks come from the second circles just added to the frontier, so their first
-// trip to memory is then an L1 hit.
-__device__ __forceinline__ void prefetch_rows(const int* srp, const int* tp, int x) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(srp + x)));
-  if (tp) asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(tp + x)));
-}
-
 // Warp 1 of the colouring CTA: while warp 0 processes its pick, load the two-hop
 // neighbourhood of the frontier's current first vertex (the likely next pick) so warp
 // 0 finds it in L1.  It only reads; the bitmap it reads is being changed by warp 0, so
 // what it finds is a hint, checked for range, and a wrong guess costs nothing but the
 // loads.  Its wait for a new pick is bounded and it stops when warp 0 is done.
 __device__ void colouring_prefetcher(int n, const int* __restrict__ srp, const int* __restrict__ sci,
-                                     const int* __restrict__ tp, const int* __restrict__ tl,
                                      const Bitmap3& bm, volatile int* hint, volatile int* done,
                                      volatile int* sink) {
   const int lane = threadIdx.x % 32;
@@ -429,13 +664,6 @@ __device__ void colouring_prefetcher(int n, const int* __restrict__ srp, const i
     }
     c = __shfl_sync(0xffffffffu, c, 0);
     if (c < 0 || c >= n) continue;
-    if (tp) {
-      const int e1 = __ldg(tp + c + 1);
-      for (int e = __ldg(tp + c) + 8 * lane; e < e1; e += 256) acc += __ldg(tl + e);
-      const int r1 = __ldg(srp + c + 1);
-      for (int q = __ldg(srp + c) + 8 * lane; q < r1; q += 256) acc += __ldg(sci + q);
-      continue;
-    }
     const int q0 = __ldg(srp + c), q1 = __ldg(srp + c + 1);
     for (int q = q0 + lane; q < q1; q += 32) {
       const int k = __ldg(sci + q);
@@ -449,8 +677,6 @@ __device__ void colouring_prefetcher(int n, const int* __restrict__ srp, const i
 // layout flags: bit 0 = frontier bitmap in shared memory, bit 1 = inV in shared memory
 __global__ void __launch_bounds__(64) colouring_kernel(int n, const int* __restrict__ srp,
                                                        const int* __restrict__ sci,
-                                                       const int* __restrict__ tp,
-                                                       const int* __restrict__ tl,
                                                        unsigned* ginV, int* wbar,
                                                        unsigned* gbitmap, int layout,
                                                        int* colour, int* meta, int max_passes) {
@@ -481,7 +707,7 @@ __global__ void __launch_bounds__(64) colouring_kernel(int n, const int* __restr
   }
   __syncthreads();
   if (threadIdx.x >= 32) {
-    colouring_prefetcher(n, srp, sci, tp, tl, bm, &s_hint, &s_done, &s_sink);
+    colouring_prefetcher(n, srp, sci, bm, &s_hint, &s_done, &s_sink);
     return;
   }
   int coloured = 0, g = 0;
@@ -542,19 +768,6 @@ __global__ void __launch_bounds__(64) colouring_kernel(int n, const int* __restr
       }
       ++coloured;
       const int q0 = __ldg(srp + v), q1 = __ldg(srp + v + 1);
-      // with two-hop lists the whole second circle is one contiguous run: its first round
-      // is loaded here, alongside the neighbours, before they leave V
-      int t0 = 0, t1 = 0;
-      int xs0[kSecondU];
-      if (tp) {
-        t0 = __ldg(tp + v);
-        t1 = __ldg(tp + v + 1);
-#pragma unroll
-        for (int u = 0; u < kSecondU; ++u) {
-          const int t = t0 + lane + 32 * u;
-          xs0[u] = t < t1 ? __ldg(tl + t) : -1;
-        }
-      }
       // Wbar = Wbar u (S_v n V), V = V / S_v  (all chunks first)
       int kb0 = 0, kl0 = 0;  // row of this lane's neighbour in the first chunk
       for (int q = q0; q < q1; q += 32) {
@@ -563,7 +776,7 @@ __global__ void __launch_bounds__(64) colouring_kernel(int n, const int* __restr
         int j = -1;
         if (qq < q1) {
           j = __ldg(sci + qq);
-          if (q == q0 && !tp) {
+          if (q == q0) {
             kb0 = __ldg(srp + j);
             kl0 = __ldg(srp + j + 1) - kb0;
           }
@@ -582,30 +795,6 @@ __global__ void __launch_bounds__(64) colouring_kernel(int n, const int* __restr
       }
       __syncwarp();
       // hat W = hat W u hat S_v: undetermined vertices of the second circle
-      if (tp) {
-#pragma unroll
-        for (int u = 0; u < kSecondU; ++u)
-          if (xs0[u] >= 0 && in_v(inV, xs0[u])) {
-            bm_set(bm, xs0[u]);
-            prefetch_rows(srp, tp, xs0[u]);
-          }
-        for (int t = t0 + 32 * kSecondU; t < t1; t += 32 * kSecondU) {
-          int xs[kSecondU];
-#pragma unroll
-          for (int u = 0; u < kSecondU; ++u) {
-            const int tt = t + lane + 32 * u;
-            xs[u] = tt < t1 ? __ldg(tl + tt) : -1;
-          }
-#pragma unroll
-          for (int u = 0; u < kSecondU; ++u)
-            if (xs[u] >= 0 && in_v(inV, xs[u])) {
-              bm_set(bm, xs[u]);
-              prefetch_rows(srp, tp, xs[u]);
-            }
-        }
-        __syncwarp();
-        continue;
-      }
       for (int q = q0; q < q1; q += 32) {
         const int qq = q + lane;
         int kb = kb0, kl = kl0;
@@ -780,38 +969,61 @@ int launch_segment_sums(int nseg, const int* seg_start, const int* src, const do
   return launch_status();
 }
 
-int launch_colouring(int n, const int* srp, const int* sci, const int* tp, const int* tl,
-                     unsigned* inV, int* wbar, unsigned* bitmap, size_t bitmap_words,
-                     int* colour, int* meta, int max_passes, cudaStream_t s) {
+int launch_colouring(int n, const int* srp, const int* sci, unsigned* inV, int* wbar,
+                     unsigned* bitmap, size_t bitmap_words, int* colour, int* meta, int max_passes,
+                     cudaStream_t s) {
   if (n <= 0) return MSP_OK;
   const int n0 = (n + 31) / 32, n1 = (n0 + 31) / 32, n2 = (n1 + 31) / 32;
   const size_t fwords = (size_t)n0 + n1 + n2;
   if (fwords > bitmap_words) return MSP_ERR_ARG;
-  const size_t cap = 220 * 1024;
   const size_t fbytes = fwords * sizeof(unsigned), vbytes = (size_t)n0 * sizeof(unsigned);
   int layout = 0;
   size_t smem = 0;
-  if (fbytes + vbytes <= cap) {
+  if (fbytes + vbytes <= kColouringSmem) {
     layout = 3;
     smem = fbytes + vbytes;
-  } else if (vbytes <= cap) {
+  } else if (vbytes <= kColouringSmem) {
     layout = 2;  // the membership tests are the hottest accesses
     smem = vbytes;
-  } else if (fbytes <= cap) {
+  } else if (fbytes <= kColouringSmem) {
     layout = 1;
     smem = fbytes;
   }
   if (smem > 0) {
-    cudaError_t e = cudaFuncSetAttribute(colouring_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
+    cudaError_t e = cudaFuncSetAttribute(
+        colouring_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColouringSmem);
     if (e != cudaSuccess) {
       layout = 0;
       smem = 0;
     }
   }
-  colouring_kernel<<<1, 64, smem, s>>>(n, srp, sci, tp, tl, inV, wbar, bitmap, layout, colour,
-                                       meta, max_passes);
+  colouring_kernel<<<1, 64, smem, s>>>(n, srp, sci, inV, wbar, bitmap, layout, colour, meta,
+                                       max_passes);
   return launch_status();
+}
+
+bool colouring_batch_ok(int n) {
+  const size_t n1 = ((size_t)n + 1023) / 1024, n2 = (n1 + 31) / 32;
+  return (n1 + n2) * sizeof(unsigned) <= 64 * 1024;
+}
+
+int launch_colouring_batch(int n, const int4* lists, const int* list, unsigned* inV, int* wbar,
+                           unsigned* bitmap, int* colour, int* meta, int max_passes,
+                           cudaStream_t s) {
+  if (n <= 0) return MSP_OK;
+  if (!colouring_batch_ok(n)) return MSP_ERR_ARG;
+  const size_t w0 = sizeof(unsigned) * (((size_t)n + 31) / 32);
+  const size_t n1 = ((size_t)n + 1023) / 1024, sum = sizeof(unsigned) * (n1 + (n1 + 31) / 32);
+  // V is read most, then the frontier's words
+  auto run = [&](auto kern, size_t smem) -> int {
+    MSP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kColouringSmem));
+    kern<<<1, 32 * kBatch, smem, s>>>(n, lists, list, inV, bitmap, wbar, colour, meta, max_passes);
+    return launch_status();
+  };
+  if (sum + 2 * w0 <= kColouringSmem) return run(colouring_batch_kernel<true, true>, sum + 2 * w0);
+  if (sum + w0 <= kColouringSmem) return run(colouring_batch_kernel<true, false>, sum + w0);
+  return run(colouring_batch_kernel<false, false>, sum);
 }
 
 }  // namespace msp

@@ -214,9 +214,8 @@ __global__ void jp_round_kernel(int n, const int* __restrict__ srp, const int* _
   }
 }
 
-// Two-hop lists of a graph for VerticesGrouping: for every vertex v the rows of its
-// neighbours, concatenated in the order of v's row (the second circle of Algorithm 4.1,
-// with repeats and with v's own neighbours, which the colouring filters out).
+// Sizes of the two-hop lists of a graph for VerticesGrouping: for every vertex v the rows of
+// its neighbours, with repeats (an upper bound of its second circle).
 __global__ void twohop_count_kernel(int n, const int* __restrict__ srp,
                                     const int* __restrict__ sci, int* __restrict__ cnt,
                                     unsigned long long* __restrict__ total) {
@@ -241,14 +240,64 @@ __global__ void twohop_count_kernel(int n, const int* __restrict__ srp,
   }
 }
 
-__global__ void twohop_fill_kernel(int n, const int* __restrict__ srp, const int* __restrict__ sci,
-                                   const int* __restrict__ tp, int* __restrict__ tl) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    int pos = tp[v];
-    for (int q = srp[v]; q < srp[v + 1]; ++q) {
-      const int k = sci[q];
-      for (int e = srp[k]; e < srp[k + 1]; ++e) tl[pos++] = sci[e];
+// Lists of VerticesGrouping, one warp per vertex: v's neighbours, then its second circle (the
+// vertices of its neighbours' rows) without repeats and without v and its neighbours; a hash
+// table in shared memory finds the repeats.  A second circle too large for the table is
+// stored as it comes (the colouring passes over what is not in V or already in the
+// frontier; it only tests more).  Place: start[v] = tp[v] + srp[v].
+constexpr int kHashSlots = 512;
+__global__ void __launch_bounds__(kThreads) twohop_lists_kernel(int n, const int* __restrict__ srp,
+                                                                const int* __restrict__ sci,
+                                                                const int* __restrict__ tp,
+                                                                const int* __restrict__ cnt,
+                                                                int4* __restrict__ meta,
+                                                                int* __restrict__ list) {
+  __shared__ int table[kThreads / 32][kHashSlots];
+  const int lane = threadIdx.x % 32;
+  int* tab = table[threadIdx.x / 32];
+  const int warps = gridDim.x * (blockDim.x / 32);
+  // true when x was not in the table yet
+  auto insert = [&](int x) {
+    unsigned h = ((unsigned)x * 2654435761u) >> 23;
+    while (true) {
+      const int old = atomicCAS(tab + h, -1, x);
+      if (old == -1) return true;
+      if (old == x) return false;
+      h = (h + 1) & (kHashSlots - 1);
     }
+  };
+  for (int v = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; v < n; v += warps) {
+    const int q0 = srp[v], deg = srp[v + 1] - q0;
+    const int start = tp[v] + q0;
+    const bool hashed = deg + cnt[v] < kHashSlots * 3 / 4;  // the table always keeps free slots
+    if (hashed) {
+      for (int k = lane; k < kHashSlots; k += 32) tab[k] = -1;
+      __syncwarp();
+      if (lane == 0) insert(v);
+    }
+    for (int q = lane; q < deg; q += 32) {
+      const int j = sci[q0 + q];
+      list[start + q] = j;
+      if (hashed) insert(j);
+    }
+    __syncwarp();
+    int pos = start + deg;
+    for (int q = 0; q < deg; ++q) {
+      const int k = sci[q0 + q], e0 = srp[k], e1 = srp[k + 1];
+      for (int e = e0; e < e1; e += 32) {
+        int x = 0;
+        bool keep = false;
+        if (e + lane < e1) {
+          x = sci[e + lane];
+          keep = !hashed || insert(x);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (keep) list[pos + __popc(m & ((1u << lane) - 1u))] = x;
+        pos += __popc(m);
+      }
+    }
+    if (lane == 0) meta[v] = make_int4(start, deg, pos - start, 0);
+    __syncwarp();
   }
 }
 
@@ -508,10 +557,11 @@ int launch_twohop_count(int n, const int* srp, const int* sci, int* cnt, unsigne
   return launch_status();
 }
 
-int launch_twohop_fill(int n, const int* srp, const int* sci, const int* tp, int* tl,
-                       cudaStream_t s) {
+int launch_twohop_lists(int n, const int* srp, const int* sci, const int* tp, const int* cnt,
+                        int4* meta, int* list, cudaStream_t s) {
   if (n <= 0) return MSP_OK;
-  twohop_fill_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(n, srp, sci, tp, tl);
+  twohop_lists_kernel<<<grid_for((size_t)n * 32, kThreads), kThreads, 0, s>>>(n, srp, sci, tp, cnt,
+                                                                             meta, list);
   return launch_status();
 }
 

@@ -48,12 +48,17 @@ int launch_segment_sums(int nseg, const int* seg_start, const int* src, const do
 // whose labels are the priority ranks (degree desc, original index asc).  scratch: inV
 // bitmap of ceil(n/32) words, n ints Wbar list, frontier bitmap words.  On return
 // colour[r] in 1..g (by label), meta[0] = g, meta[1] = error flag (a bounded loop ran
-// out).  tp/tl: the graph's two-hop lists (launch_twohop_*), or both nullptr.
-// max_passes: passes of Algorithm 4.2 (colours) before the loop gives up (n always
+// out).  max_passes: passes of Algorithm 4.2 (colours) before the loop gives up (n always
 // suffices: every pass colours at least one vertex).
-int launch_colouring(int n, const int* srp, const int* sci, const int* tp, const int* tl,
-                     unsigned* inV, int* wbar, unsigned* bitmap, size_t bitmap_words,
-                     int* colour, int* meta, int max_passes, cudaStream_t s);
+int launch_colouring(int n, const int* srp, const int* sci, unsigned* inV, int* wbar,
+                     unsigned* bitmap, size_t bitmap_words, int* colour, int* meta, int max_passes,
+                     cudaStream_t s);
+// the same from the lists of launch_twohop_lists, several picks per search and per trip to
+// memory; for the graph sizes of colouring_batch_ok
+bool colouring_batch_ok(int n);
+int launch_colouring_batch(int n, const int4* lists, const int* list, unsigned* inV, int* wbar,
+                           unsigned* bitmap, int* colour, int* meta, int max_passes,
+                           cudaStream_t s);
 
 // ---- other setup kernels (setup_kernels.cu) ----
 // errors in the BSR pattern: row pointers outside [0, nnz] or decreasing, unsorted / out
@@ -82,12 +87,14 @@ int launch_jp_keys(int n, const int* srp, unsigned long long seed, unsigned long
 // coloured, counters[1] = max(counters[1], colour)
 int launch_jp_round(int n, const int* srp, const int* sci, const int* rank, int* colour,
                     int* counters, cudaStream_t s);
-// two-hop lists of a graph (srp/sci): cnt[v] = sum over the neighbours k of v of deg(k),
-// *total = their sum; then tl[tp[v] ...] = the neighbours' rows concatenated in row order
+// cnt[v] = sum over the neighbours k of v of deg(k), *total = their sum
 int launch_twohop_count(int n, const int* srp, const int* sci, int* cnt, unsigned long long* total,
                         cudaStream_t s);
-int launch_twohop_fill(int n, const int* srp, const int* sci, const int* tp, int* tl,
-                       cudaStream_t s);
+// lists of the batched colouring: vertex v's neighbours and then its second circle at
+// list[start], start = tp[v] + srp[v] (tp: exclusive sums of cnt); meta[v] = (start, deg,
+// entries, 0)
+int launch_twohop_lists(int n, const int* srp, const int* sci, const int* tp, const int* cnt,
+                        int4* meta, int* list, cudaStream_t s);
 // ELL copy (K slots per row, slot k of row i at i*K + k) of the off-diagonal entries of a
 // CSR level matrix; meta[i] = count | (entries left of the diagonal) << 16, or -1 for rows
 // longer than K (their slots hold (i, 0)); diag[i] = a_ii
