@@ -139,7 +139,8 @@ int launch_reduce_partials_strided(int K, int nblocks, int stride, const double*
 // *p = v in stream order (a kernel, so that it never waits behind host copies)
 int launch_set_int(int* p, int v, cudaStream_t s);
 // partial[b * stride + k] = block b's share of V_k . x, k < K; with jsel (device index j),
-// K = j + 1 and x = V_j at run time (nothing when j < 0); stride <= kKrylovMaxK
+// K = j + 1 and x = V_j at run time (nothing when j < 0); stride <= kKrylovMaxK; without jsel
+// nblocks = multi_dot_blocks(n, K)
 int launch_multi_dot1(size_t n, const double* V, size_t ldv, int K, const double* x,
                       double* partial, int stride, int nblocks, cudaStream_t s,
                       const int* jsel = nullptr);
@@ -176,7 +177,9 @@ int launch_gather_blocks(int nb, int b, const int* perm, const double* in, doubl
 int launch_scatter_blocks(int nb, int b, const int* perm, const double* in, double* out,
                           cudaStream_t s);
 
-int krylov_blocks();  // number of blocks the reduction kernels use
+int krylov_blocks();              // most blocks the reduction kernels use
+int krylov_blocks_for(size_t n);  // blocks of the norms and updates of vectors of n elements
+int multi_dot_blocks(size_t n, int K);  // blocks (per group of vectors) of K dot products
 
 // ---------------- batched Krylov over a block-diagonal system ----------------
 // Chunks of the (colour-ordered) vector, each inside one instance: chunk c covers the

@@ -1167,7 +1167,7 @@ int basis_dot(msp_handle h, cudaStream_t s, bool branch) {
   // levels, and leaving most of each SM's registers to the sweeps it runs beside (measured
   // on the 1.12M-row system: 166.5 ms per solve, against 178.7 with one block per SM and
   // 171.3 with four)
-  const int nbk = std::min(krylov_blocks(), sm_count() * 2);
+  const int nbk = std::min(krylov_blocks_for(n), sm_count() * 2);
   {
     Probe pr("krylov_basis_dot", 0.0, d);  // bytes are counted by the caller (j is known there)
     MSP_TRY(launch_multi_dot1(n, h->V.p, n, 0, nullptr, h->partial_u.p, kKrylovMaxK, nbk, d,
@@ -1634,7 +1634,7 @@ int alloc_work(msp_handle h) {
 
 // ||x||_2 of a device vector (deterministic reduction), synchronous
 int norm2(msp_handle h, const double* x, size_t n, double* out, cudaStream_t s) {
-  const int nbk = krylov_blocks();
+  const int nbk = krylov_blocks_for(n);
   MSP_TRY(launch_norm2_partial(n, x, h->partial.p, nbk, s));
   MSP_TRY(launch_reduce_partials(1, nbk, h->partial.p, h->nrm.p, false, s));
   MSP_CUDA_TRY(cudaMemcpyAsync(h->h_pin, h->nrm.p, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1661,7 +1661,7 @@ int fgmres(msp_handle h, double tol, int* iters, double* relres, double* relres_
   NvtxRange nvtx("msp:fgmres");
   const size_t n = (size_t)h->nb * h->b;
   const int m = h->cfg.restart;
-  const int nbk = krylov_blocks();
+  const int nbk = krylov_blocks_for(n);
   const double* bvec = h->bperm.p;
   double* x = h->xperm.p;
   double* V = h->V.p;
@@ -1778,9 +1778,11 @@ int fgmres(msp_handle h, double tol, int* iters, double* relres, double* relres_
       const int K = j + 2;  // u_0 .. u_j and w
       {
         Probe pr("krylov_multi_dot", (double)(K + 1) * n * 8.0, s, 1, 2.0 * K * n);
-        MSP_TRY(launch_multi_dot1(n, V, n, K, w, h->partial.p, kKrylovMaxK, nbk, s));
+        MSP_TRY(launch_multi_dot1(n, V, n, K, w, h->partial.p, kKrylovMaxK,
+                                  multi_dot_blocks(n, K), s));
       }
-      MSP_TRY(launch_reduce_partials_strided(K, nbk, kKrylovMaxK, h->partial.p, h->gs_d.p + K,
+      MSP_TRY(launch_reduce_partials_strided(K, multi_dot_blocks(n, K), kKrylovMaxK, h->partial.p,
+                                             h->gs_d.p + K,
                                              s));
       MSP_TRY(launch_dcgs_coef(j, h->gs_d.p, T, ldt, h->gs_g.p, out, s));
       {
@@ -1830,9 +1832,11 @@ int fgmres(msp_handle h, double tol, int* iters, double* relres, double* relres_
         // column j final now: column j + 1 of T from the dot products of u_{j+1}
         {
           Probe pr("krylov_finalize_dot", (double)(j + 2) * n * 8.0, s, 1, 2.0 * (j + 2) * n);
-          MSP_TRY(launch_multi_dot1(n, V, n, j + 2, w, h->partial.p, kKrylovMaxK, nbk, s));
+          MSP_TRY(launch_multi_dot1(n, V, n, j + 2, w, h->partial.p, kKrylovMaxK,
+                                    multi_dot_blocks(n, j + 2), s));
         }
-        MSP_TRY(launch_reduce_partials(j + 2, nbk, h->partial.p, h->gs_d.p, false, s));
+        MSP_TRY(launch_reduce_partials(j + 2, multi_dot_blocks(n, j + 2), h->partial.p, h->gs_d.p,
+                                       false, s));
         MSP_TRY(launch_dcgs_finalize(j + 1, h->gs_d.p, T, ldt, out, s));
         MSP_TRY(fetch_out());
         if (!std::isfinite(hp[145])) return MSP_ERR_NONFINITE;
@@ -1881,8 +1885,13 @@ int fgmres(msp_handle h, double tol, int* iters, double* relres, double* relres_
 
 // Chunks of the batched Krylov kernels: level-0 colour classes hold the rows of every
 // instance in increasing original index, i.e. instance by instance, so the vector splits
-// into (colour, instance) segments, cut into chunks of at most kSegChunk elements.
-constexpr int kSegChunk = 8192;
+// into (colour, instance) segments, cut into chunks.  A chunk is one block's work: eight per
+// SM, between 1024 elements (below, a block's reductions cost more than its products) and
+// 8192.  24 instances of 6k cells, b = 4, with 8192 always: one chunk per SM and the dot
+// products 116 us a step, now 48; the updates 75 us, now 19.
+int seg_chunk(size_t n) {
+  return (int)std::min<size_t>(8192, std::max<size_t>(1024, n / ((size_t)sm_count() * 8) / 256 * 256));
+}
 constexpr int kBatchOut = 160;  // per-instance results of a Gram-Schmidt step (see dcgs_coef_kernel)
 
 SegChunks seg_chunks(msp_handle h) {
@@ -2675,6 +2684,7 @@ int msp_set_instances(msp_handle h, int32_t count, const int32_t* h_row_offsets)
     MSP_CUDA_TRY(cudaMemcpy(perm.data(), h->perm0.p, sizeof(int) * (size_t)nb,
                             cudaMemcpyDeviceToHost));
     std::vector<int> cstart, cend, cinst;
+    const int chunk = seg_chunk((size_t)nb * b);
     const std::vector<int> offs(h_row_offsets, h_row_offsets + count + 1);
     auto inst_of = [&](int r) {
       return (int)(std::upper_bound(offs.begin(), offs.end(), r) - offs.begin()) - 1;
@@ -2687,9 +2697,9 @@ int msp_set_instances(msp_handle h, int32_t count, const int32_t* h_row_offsets)
         int q = p + 1;
         while (q < p1 && inst_of(perm[q]) == inst) ++q;
         if (q < p1 && inst_of(perm[q]) < inst) return MSP_ERR_PATTERN;  // not instance-major
-        for (long long e = (long long)p * b; e < (long long)q * b; e += kSegChunk) {
+        for (long long e = (long long)p * b; e < (long long)q * b; e += chunk) {
           cstart.push_back((int)e);
-          cend.push_back((int)std::min<long long>(e + kSegChunk, (long long)q * b));
+          cend.push_back((int)std::min<long long>(e + chunk, (long long)q * b));
           cinst.push_back(inst);
         }
         p = q;

@@ -1062,11 +1062,14 @@ __device__ __forceinline__ double transpose_sum8(double (&a)[8], int lane) {
 __global__ void set_int_kernel(int* __restrict__ p, int v) { *p = v; }
 
 // One right-hand vector, four elements in flight per thread: partial[b * stride + k] =
-// V_k . x over block b's share, k < K.  With `jsel` (a device index j, read at run time) the
-// kernel takes K = j + 1 and x = V_j, the basis against its newest vector, so that one
-// captured launch serves every step; j < 0 makes it return at once.  The basis is read
-// with evict-first loads: it is streamed once, and the kernel may run beside other work
-// whose data should stay in L2.
+// V_k . x over block b's share, k < K.  The vectors are dealt over gridDim.y blocks of at most
+// 8 each, all of about the same number, so that a block reduces its sums once and no
+// block is left with a chunk of one vector (132k x 4 unknowns, 50 steps, mean of 17
+// vectors: 37.8 us a launch with the chunks in turn, 24.6 now; 1.12M x 4: 170 and 136 us).  With `jsel` (a device
+// index j, read at run time) the kernel takes K = j + 1 and x = V_j, the basis against its
+// newest vector, in chunks of 8 (gridDim.y = 1), so that one captured launch serves every
+// step; j < 0 makes it return at once.  The basis is read with evict-first loads: it is
+// streamed once, and the kernel may run beside other work whose data should stay in L2.
 __global__ void __launch_bounds__(kThreads) multi_dot1_kernel(size_t n, const double* __restrict__ V,
                                                              size_t ldv, int K,
                                                              const double* __restrict__ x,
@@ -1081,10 +1084,12 @@ __global__ void __launch_bounds__(kThreads) multi_dot1_kernel(size_t n, const do
     K = j + 1;
     x = V + (size_t)j * ldv;
   }
+  const int per = gridDim.y > 1 ? (K + (int)gridDim.y - 1) / (int)gridDim.y : kDotChunk;
+  const int kend = gridDim.y > 1 ? min(K, ((int)blockIdx.y + 1) * per) : K;
   const int lane = threadIdx.x % kWarp, wid = threadIdx.x / kWarp;
   const int slot = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-  for (int k0 = 0; k0 < K; k0 += kDotChunk) {
-    const int kc = min(kDotChunk, K - k0);
+  for (int k0 = (int)blockIdx.y * per; k0 < kend; k0 += per) {
+    const int kc = min(per, kend - k0);
     double a[kDotChunk];
 #pragma unroll
     for (int k = 0; k < kDotChunk; ++k) a[k] = 0.0;
@@ -1104,11 +1109,21 @@ __global__ void __launch_bounds__(kThreads) multi_dot1_kernel(size_t n, const do
           for (int q = 0; q < 4; ++q) a[k] = fma(vk[q], u[q], a[k]);
         }
     }
-    for (; i < n; i += G) {
-      const double u = x[i];
+    if (i < n) {  // up to three elements more, in flight together as well
+      double u[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) u[q] = i + q * G < n ? x[i + q * G] : 0.0;
 #pragma unroll
       for (int k = 0; k < kDotChunk; ++k)
-        if (k < kc) a[k] = fma(__ldcs(V + (size_t)(k0 + k) * ldv + i), u, a[k]);
+        if (k < kc) {
+          double vk[3];
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+            vk[q] = i + q * G < n ? __ldcs(V + (size_t)(k0 + k) * ldv + i + q * G) : 0.0;
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+            if (i + q * G < n) a[k] = fma(vk[q], u[q], a[k]);
+        }
     }
     const double r = transpose_sum8(a, lane);
     __syncthreads();  // the previous chunk's reads of sh are done
@@ -1331,6 +1346,38 @@ __global__ void reduce_partials_kernel(int K, int nblocks, const double* __restr
   if (lane == 0) out[k] = accumulate ? out[k] + s : s;
 }
 
+// w_i -= sum_k hs[k] V_k[i] for i = i0, i0 + G, ... < n; the sum of the new w_i^2.  Two
+// elements at a time, so that their chains of K dependent FMAs overlap, then one; no test
+// inside the loops over k (four elements under tests took 282 us against 133 us on 1.12M x 4).
+__device__ __forceinline__ double axpy_norm(size_t i0, size_t n, size_t G,
+                                            const double* __restrict__ V, size_t ldv, int K,
+                                            const double* hs, double* __restrict__ w) {
+  double nrm = 0.0;
+  size_t i = i0;
+  for (; i + G < n; i += 2 * G) {
+    double w0 = w[i], w1 = w[i + G];
+    const double* v = V + i;
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+      const double h = -hs[k];
+      w0 = fma(h, __ldg(v + (size_t)k * ldv), w0);
+      w1 = fma(h, __ldg(v + (size_t)k * ldv + G), w1);
+    }
+    w[i] = w0;
+    w[i + G] = w1;
+    nrm = fma(w0, w0, nrm);
+    nrm = fma(w1, w1, nrm);
+  }
+  if (i < n) {
+    double wi = w[i];
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) wi = fma(-hs[k], __ldg(V + (size_t)k * ldv + i), wi);
+    w[i] = wi;
+    nrm = fma(wi, wi, nrm);
+  }
+  return nrm;
+}
+
 __global__ void __launch_bounds__(kThreads) multi_axpy_norm_kernel(
     size_t n, const double* __restrict__ V, size_t ldv, int K, const double* __restrict__ h,
     double* __restrict__ w, double* __restrict__ partial, const int* __restrict__ gate) {
@@ -1339,14 +1386,8 @@ __global__ void __launch_bounds__(kThreads) multi_axpy_norm_kernel(
   if (gate && *gate == 0) return;
   for (int k = threadIdx.x; k < K; k += blockDim.x) hs[k] = h[k];
   __syncthreads();
-  double nrm = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    double wi = w[i];
-    for (int k = 0; k < K; ++k) wi = fma(-hs[k], __ldg(V + (size_t)k * ldv + i), wi);
-    w[i] = wi;
-    nrm = fma(wi, wi, nrm);
-  }
+  const size_t G = (size_t)gridDim.x * blockDim.x;
+  const double nrm = axpy_norm(blockIdx.x * (size_t)blockDim.x + threadIdx.x, n, G, V, ldv, K, hs, w);
   double t = block_sum(nrm, sh);
   if (threadIdx.x == 0) partial[(size_t)blockIdx.x * kMaxK] = t;
 }
@@ -1462,14 +1503,21 @@ __global__ void __launch_bounds__(kThreads) seg_multi_dot2_kernel(
       double a0[kDotChunk], a1[kDotChunk];
 #pragma unroll
       for (int k = 0; k < kDotChunk; ++k) a0[k] = a1[k] = 0.0;
-      for (size_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        const double u = x0[i], w = x1[i];
+      for (size_t i = i0 + threadIdx.x; i < i1; i += 2 * blockDim.x) {  // two elements in flight
+        const size_t i2 = i + blockDim.x;
+        const bool two = i2 < i1;
+        const double u = x0[i], w = x1[i], u2 = two ? x0[i2] : 0.0, w2 = two ? x1[i2] : 0.0;
 #pragma unroll
         for (int k = 0; k < kDotChunk; ++k)
           if (k < kc) {
-            const double vk = __ldg(V + (size_t)(k0 + k) * ldv + i);
+            const double* vp = V + (size_t)(k0 + k) * ldv;
+            const double vk = __ldg(vp + i), vk2 = two ? __ldg(vp + i2) : 0.0;
             a0[k] = fma(vk, u, a0[k]);
             a1[k] = fma(vk, w, a1[k]);
+            if (two) {
+              a0[k] = fma(vk2, u2, a0[k]);
+              a1[k] = fma(vk2, w2, a1[k]);
+            }
           }
       }
       const double r0 = transpose_sum8(a0, lane);
@@ -1543,13 +1591,7 @@ __global__ void __launch_bounds__(kThreads) seg_multi_axpy_norm_kernel(
     __syncthreads();  // the previous chunk's reads of hs are done
     for (int k = threadIdx.x; k < K; k += blockDim.x) hs[k] = coef[(size_t)inst * kMaxK + k];
     __syncthreads();
-    double nrm = 0.0;
-    for (size_t i = cs[c] + threadIdx.x; i < (size_t)ce[c]; i += blockDim.x) {
-      double wi = w[i];
-      for (int k = 0; k < K; ++k) wi = fma(-hs[k], __ldg(V + (size_t)k * ldv + i), wi);
-      w[i] = wi;
-      nrm = fma(wi, wi, nrm);
-    }
+    const double nrm = axpy_norm((size_t)cs[c] + threadIdx.x, (size_t)ce[c], blockDim.x, V, ldv, K, hs, w);
     const double t = block_sum(nrm, sh);
     if (threadIdx.x == 0) partial[(size_t)c * kMaxK] = t;
   }
@@ -2023,6 +2065,18 @@ int launch_cast_f2d(size_t n, const float* in, double* out, cudaStream_t s) {
 
 int krylov_blocks() { return sm_count() * 4; }
 
+// blocks for vectors of n elements: two elements a thread on small ones (more blocks would
+// only lengthen the sum of the partials)
+int krylov_blocks_for(size_t n) {
+  return (int)std::min<size_t>((size_t)krylov_blocks(), std::max<size_t>(1, (n + 511) / 512));
+}
+
+// the share of each of the ceil(K / 8) groups of vectors of a dot-product launch
+int multi_dot_blocks(size_t n, int K) {
+  const int groups = std::max(1, (K + kDotChunk - 1) / kDotChunk);
+  return std::max(1, std::min(krylov_blocks_for(n), krylov_blocks() / groups));
+}
+
 int launch_reduce_partials_strided(int K, int nblocks, int stride, const double* partial,
                                    double* out, cudaStream_t s, int* jsel) {
   if (jsel) {  // one block: its threads all read the index before it moves on
@@ -2048,7 +2102,9 @@ int launch_multi_dot1(size_t n, const double* V, size_t ldv, int K, const double
                       double* partial, int stride, int nblocks, cudaStream_t s, const int* jsel) {
   if (stride > kMaxK || (!jsel && (K > stride || !x))) return MSP_ERR_ARG;
   if (!jsel && K <= 0) return MSP_OK;
-  multi_dot1_kernel<<<nblocks, kThreads, 0, s>>>(n, V, ldv, K, x, partial, stride, jsel);
+  const int groups = jsel ? 1 : (K + kDotChunk - 1) / kDotChunk;
+  multi_dot1_kernel<<<dim3(nblocks, groups), kThreads, 0, s>>>(n, V, ldv, K, x, partial, stride,
+                                                               jsel);
   return launch_status();
 }
 
