@@ -57,6 +57,15 @@ constexpr int kZeroExp = -4000;                           // exponent of an all-
 
 inline int launch_status() { return launch_check(__FILE__, __LINE__); }
 
+// The dense matrices are stored by tiles of 128 rows x 32 columns (row tiles of `nct` column
+// tiles), a tile by pairs of columns, then rows: the 32 rows that a warp of the products'
+// epilogue holds are 512 consecutive bytes.  (With rows of the whole matrix each lane
+// touched its own line: 2.7 times the sectors, n = 9,836 157 -> LAYFIG ms.)
+__device__ __forceinline__ size_t tile_at(int nct, int i, int j) {
+  return ((size_t)(i / kRowTile) * nct + j / kColTile) * (kRowTile * kColTile) +
+         (size_t)((j % kColTile) / 2) * (2 * kRowTile) + (i % kRowTile) * 2 + (j & 1);
+}
+
 __device__ void raise_flag(DevFlags* f, int code, int index) {
   if (atomicCAS(&f->code, MSP_OK, code) == MSP_OK) f->index = index;
 }
@@ -116,9 +125,9 @@ __device__ __forceinline__ void store_digits8(const double (&x)[8], int e, char*
 }
 
 // Digits of the rows of a tile of 32 rows of A[:, k0..k0+96) (A padded: whole tiles exist),
-// and the row exponents.  With Y the rows [z0, z1) are taken as zeros, and Y (kP values a
-// row) receives A[:, k0..k0+96) with -I in the rows [z0, z1).
-__global__ void __launch_bounds__(256) slice_rows_kernel(int lda, int k0, int z0, int z1,
+// and the row exponents.  With Y the rows [z0, z1) are taken as zeros, and Y (96 columns)
+// receives A[:, k0..k0+96) with -I in the rows [z0, z1).
+__global__ void __launch_bounds__(256) slice_rows_kernel(int nct, int k0, int z0, int z1,
                                                          const double* __restrict__ A,
                                                          char* __restrict__ S,
                                                          int* __restrict__ exps,
@@ -126,12 +135,18 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(int lda, int k0, int z0
   __shared__ double sh[32][kP + 1];
   __shared__ int se[32];
   const int r0 = blockIdx.x * 32;
-  for (int t = threadIdx.x; t < 32 * kP; t += 256) {
-    const int r = t / kP, q = t % kP, i = r0 + r;
+#pragma unroll
+  for (int t = threadIdx.x; t < 32 * (kP / 2); t += 256) {
+    const int r = t % 32, q = t / 32 * 2, i = r0 + r;
     const bool z = Y && i >= z0 && i < z1;
-    const double x = z ? 0.0 : A[(size_t)i * lda + k0 + q];
-    sh[r][q] = x;
-    if (Y) Y[(size_t)i * kP + q] = z ? (i - z0 == q ? -1.0 : 0.0) : x;
+    double2 x = make_double2(0.0, 0.0);
+    if (!z) x = *reinterpret_cast<const double2*>(A + tile_at(nct, i, k0 + q));
+    sh[r][q] = x.x;
+    sh[r][q + 1] = x.y;
+    if (Y) {
+      if (z) x = make_double2(i - z0 == q ? -1.0 : 0.0, i - z0 == q + 1 ? -1.0 : 0.0);
+      *reinterpret_cast<double2*>(Y + tile_at(kKTiles, i, q)) = x;
+    }
   }
   __syncthreads();
   {
@@ -176,7 +191,7 @@ constexpr int kDigitStrideB = (kColTile / 8) * 128;
 // The panel's row exchanges on a tile of 32 columns of A, and the digits of the exchanged
 // rows K (T, for the tiles of K the block A_KK).  perm[0] = number of rows that change, then pairs
 // (destination, source); the K rows of T are read after the exchange.
-__global__ void __launch_bounds__(256) swap_slice_kernel(int lda, int k0, int kb,
+__global__ void __launch_bounds__(256) swap_slice_kernel(int nct, int k0, int kb,
                                                          double* __restrict__ A,
                                                          const int* __restrict__ perm,
                                                          char* __restrict__ S,
@@ -191,13 +206,18 @@ __global__ void __launch_bounds__(256) swap_slice_kernel(int lda, int k0, int kb
   const int cnt = perm[0];
   for (int t = w; t < cnt; t += 8) {
     if (lane == 0) sd[t] = perm[1 + 2 * t];
-    sh[t][lane] = A[(size_t)perm[2 + 2 * t] * lda + c0 + lane];
+    sh[t][lane] = A[tile_at(nct, perm[2 + 2 * t], c0 + lane)];
   }
   __syncthreads();
-  for (int t = w; t < cnt; t += 8) A[(size_t)sd[t] * lda + c0 + lane] = sh[t][lane];
+  for (int t = w; t < cnt; t += 8) A[tile_at(nct, sd[t], c0 + lane)] = sh[t][lane];
   __syncthreads();  // the rows K below are read back by the block that wrote them
-  for (int q = w; q < kP; q += 8)
-    sh[q][lane] = q < kb ? A[(size_t)(k0 + q) * lda + c0 + lane] : 0.0;
+  for (int t = threadIdx.x; t < kP * (kColTile / 2); t += 256) {
+    const int q = t % kP, c = t / kP * 2;
+    double2 x = make_double2(0.0, 0.0);
+    if (q < kb) x = *reinterpret_cast<const double2*>(A + tile_at(nct, k0 + q, c0 + c));
+    sh[q][c] = x.x;
+    sh[q][c + 1] = x.y;
+  }
   __syncthreads();
   double m = 0.0;
   bool bad = false;
@@ -228,12 +248,15 @@ __global__ void __launch_bounds__(256) swap_slice_kernel(int lda, int k0, int kb
 
 // ------------------------------------------------------------------ LU of the panel copy
 // X[i][c] = A[k0 + i][k0 + c] for the rows below k0, columns past kb zero
-__global__ void panel_copy_kernel(int m, int k0, int kb, int lda, const double* __restrict__ A,
+__global__ void panel_copy_kernel(int m, int k0, int kb, int nct, const double* __restrict__ A,
                                   double* __restrict__ X) {
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)m * kP;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)m * (kP / 2);
        t += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t / kP), c = (int)(t % kP);
-    X[t] = c < kb ? A[(size_t)(k0 + i) * lda + k0 + c] : 0.0;
+    const int i = (int)(t % m), c = (int)(t / m) * 2;
+    double2 x = *reinterpret_cast<const double2*>(A + tile_at(nct, k0 + i, k0 + c));
+    if (c >= kb) x.x = 0.0;
+    if (c + 1 >= kb) x.y = 0.0;
+    *reinterpret_cast<double2*>(X + (size_t)i * kP + c) = x;
   }
 }
 
@@ -736,9 +759,10 @@ __device__ __forceinline__ double add_digits(const float (&S)[kGroups], int e, d
   return fma(dl, fl, fma(dh, fh, c));
 }
 
-// One product of a step on the tiles (128 x 32) of C (leading dimension ldc), V = SA SB:
-//   kUpdate: C = A, the columns outside K (kt0: the first tile of K, 3 tiles left out):
-//            C += V, or C = V for the rows K;
+// One product of a step on the tiles (128 x 32) of C (row tiles of ctiles column tiles; the
+// product's first column tile is coff), V = SA SB:
+//   kUpdate: C = A, the nct column tiles from cbegin, without the kskip tiles from kt0 on (the
+//            columns K and those done by another launch): C += V, or C = V for the rows K;
 //   kFirst:  C = the columns K: C = -V, or D for the rows K;
 //   kResid:  C += V;  kCorrect: C -= V (both on 96 columns).
 enum Product { kUpdate, kFirst, kResid, kCorrect };
@@ -753,7 +777,8 @@ constexpr int kEpiCols = kColTile / (kEpiWarps / 4);  // columns of a tile per e
 constexpr size_t kGemmSmem = kTileA + kStages * kChunkB + 512;
 template <Product kMode>
 __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
-    int ldc, int k0, int kb, int nrt, int nct, int kt0, double* __restrict__ C,
+    int ctiles, int coff, int k0, int kb, int nrt, int nct, int cbegin, int kt0, int kskip,
+    double* __restrict__ C,
     const char* __restrict__ SA, const int* __restrict__ ea, const char* __restrict__ SB,
     const int* __restrict__ eb, const double* __restrict__ D, DevFlags* flags) {
   extern __shared__ __align__(128) char sm[];
@@ -801,7 +826,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
       bool run = true;
       for (long long t = t0; t < t1 && run; ++t) {
         const int rt = (int)(t / nct), q = (int)(t % nct);
-        const int ct = kMode != kUpdate ? q : q + (q >= kt0 ? kKTiles : 0);
+        const int ct = kMode != kUpdate ? q : cbegin + q + (q >= kt0 ? kskip : 0);
         if (rt != prev) {
           // the previous row tile's digits are free once its last chunk has been used
           if (g > 0)
@@ -865,19 +890,24 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
   } else {
     const int quad = wid & 3, part = wid >> 2;  // a warp reads the TMEM lanes of its quadrant
     constexpr double sign = kMode == kFirst || kMode == kCorrect ? -1.0 : 1.0;
+    // this thread's first pair of columns in a tile of C
+    auto c_pairs = [&](int rt, int ct) {
+      return C + ((size_t)rt * ctiles + coff + ct) * (kRowTile * kColTile) +
+             (size_t)(part * kEpiCols / 2) * (2 * kRowTile) + (quad * 32 + lane) * 2;
+    };
     // what a tile's C starts from: the rows' and columns' values, loaded one tile ahead
     auto load_c = [&](long long t, double (&cv)[kEpiCols]) {
       const int rt = (int)(t / nct), q = (int)(t % nct);
-      const int ct = kMode != kUpdate ? q : q + (q >= kt0 ? kKTiles : 0);
+      const int ct = kMode != kUpdate ? q : cbegin + q + (q >= kt0 ? kskip : 0);
       const int i = rt * kRowTile + quad * 32 + lane;
       const bool in_k = i >= k0 && i < k0 + kb;
       const int cb = ct * kColTile + part * kEpiCols;
-      const double* src = kMode == kFirst ? D + (size_t)(i - k0) * kP + cb
-                                          : C + (size_t)i * ldc + cb;
+      const double* src = kMode == kFirst ? D + (size_t)(i - k0) * kP + cb : c_pairs(rt, ct);
+      constexpr int pitch = kMode == kFirst ? 2 : 2 * kRowTile;  // between pairs of columns
       const bool use = kMode == kFirst ? in_k : kMode != kUpdate || !in_k;
 #pragma unroll
       for (int p = 0; p < kEpiCols / 2; ++p) {
-        const double2 v = use ? *reinterpret_cast<const double2*>(src + 2 * p)
+        const double2 v = use ? *reinterpret_cast<const double2*>(src + p * pitch)
                               : make_double2(0.0, 0.0);
         cv[2 * p] = v.x;
         cv[2 * p + 1] = v.y;
@@ -888,11 +918,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
     if (t0 < t1) load_c(t0, cn);
     for (long long t = t0; t < t1; ++t, ++it) {
       const int rt = (int)(t / nct), q = (int)(t % nct);
-      const int ct = kMode != kUpdate ? q : q + (q >= kt0 ? kKTiles : 0);
+      const int ct = kMode != kUpdate ? q : cbegin + q + (q >= kt0 ? kskip : 0);
       const int i = rt * kRowTile + quad * 32 + lane;
       const bool in_k = i >= k0 && i < k0 + kb;
       const int cb = ct * kColTile + part * kEpiCols;
-      double* crow = C + (size_t)i * ldc + cb;
+      double* cpair = c_pairs(rt, ct);
       double cv[kEpiCols];
 #pragma unroll
       for (int p = 0; p < kEpiCols; ++p) cv[p] = cn[p];
@@ -930,7 +960,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
       }
 #pragma unroll
       for (int p = 0; p < kEpiCols / 2; ++p)
-        *reinterpret_cast<double2*>(crow + 2 * p) = make_double2(cv[2 * p], cv[2 * p + 1]);
+        *reinterpret_cast<double2*>(cpair + p * 2 * kRowTile) = make_double2(cv[2 * p], cv[2 * p + 1]);
     }
   }
   __syncthreads();
@@ -953,23 +983,30 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-__global__ void csr_to_dense_kernel(int n, int lda, const int* __restrict__ rp,
+__global__ void csr_to_dense_kernel(int n, int nct, const int* __restrict__ rp,
                                     const int* __restrict__ ci, const double* __restrict__ v,
                                     double* __restrict__ A) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double* row = A + (size_t)i * lda;
-    for (int p = rp[i]; p < rp[i + 1]; ++p) row[ci[p]] = v[p];
+    for (int p = rp[i]; p < rp[i + 1]; ++p) A[tile_at(nct, i, ci[p])] = v[p];
   }
 }
 
-// out (n x n) = A with its columns in the order colperm
-__global__ void unscramble_kernel(int n, int lda, const int* __restrict__ colperm,
-                                  const double* __restrict__ A, double* __restrict__ out) {
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)n * n;
-       t += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t / n), c = (int)(t % n);
-    out[t] = A[(size_t)i * lda + colperm[c]];
-  }
+// out (n x n, row-major) = A with its columns in the order colperm: 32 x 32 pieces through
+// shared memory, read along the rows of A's tiles and written along those of out
+__global__ void __launch_bounds__(256) unscramble_kernel(int n, int nct,
+                                                         const int* __restrict__ colperm,
+                                                         const double* __restrict__ A,
+                                                         double* __restrict__ out) {
+  __shared__ double sh[32][33];
+  const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
+  const int i0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+#pragma unroll
+  for (int c = w; c < 32; c += 8)
+    sh[lane][c] = (i0 + lane < n && c0 + c < n) ? A[tile_at(nct, i0 + lane, colperm[c0 + c])] : 0.0;
+  __syncthreads();
+#pragma unroll
+  for (int r = w; r < 32; r += 8)
+    if (i0 + r < n && c0 + lane < n) out[(size_t)(i0 + r) * n + c0 + lane] = sh[r][lane];
 }
 
 // The sub-panels of one step: LU of the m x kb panel copy X.
@@ -1006,13 +1043,41 @@ int lu_panel(int m, int kb, int k0, double* X, int* piv, DevFlags* flags, cudaSt
   return MSP_OK;
 }
 
+// A stream of its own for the panels (of high priority, so that a panel's cluster is placed
+// before the update's blocks), joined before it goes
+struct SideStream {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t ready = nullptr, copied = nullptr, factored = nullptr;
+  SideStream() = default;
+  SideStream(const SideStream&) = delete;
+  SideStream& operator=(const SideStream&) = delete;
+  int create() {
+    int least = 0, greatest = 0;
+    MSP_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    MSP_CUDA_TRY(cudaStreamCreateWithPriority(&stream, cudaStreamNonBlocking, greatest));
+    MSP_CUDA_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+    MSP_CUDA_TRY(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming));
+    MSP_CUDA_TRY(cudaEventCreateWithFlags(&factored, cudaEventDisableTiming));
+    return MSP_OK;
+  }
+  ~SideStream() {
+    if (stream) {
+      cudaStreamSynchronize(stream);
+      cudaStreamDestroy(stream);
+    }
+    if (ready) cudaEventDestroy(ready);
+    if (copied) cudaEventDestroy(copied);
+    if (factored) cudaEventDestroy(factored);
+  }
+};
+
 }  // namespace
 
 int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v, double* out,
                            DevFlags* flags, cudaStream_t s) {
   if (n <= 0) return MSP_ERR_ARG;
   const int lda = (int)(div_up(n, kP) * kP), nrt = (int)div_up(n, kRowTile);
-  const int nct = (int)div_up(n, kColTile);
+  const int nct = (int)div_up(n, kColTile), act = lda / kColTile;  // column tiles used, stored
   const size_t rows = (size_t)nrt * kRowTile;
   DevBuf<double> A, X, Y, D;
   DevBuf<char> SA, ST, SD;
@@ -1032,7 +1097,7 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
   MSP_TRY(perm.alloc(1 + 4 * kP));
   MSP_TRY(cols_d.alloc(n));
   MSP_CUDA_TRY(cudaMemsetAsync(A.p, 0, rows * lda * sizeof(double), s));
-  csr_to_dense_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, lda, rp, ci, v, A.p);
+  csr_to_dense_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, act, rp, ci, v, A.p);
   MSP_TRY(launch_status());
   const size_t diag_smem = sizeof(double) * (kP * (kP + 1) + kP);
   MSP_CUDA_TRY(cudaFuncSetAttribute(diag_inverse_panel_kernel,
@@ -1045,57 +1110,83 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
   MSP_CUDA_TRY(cudaFuncSetAttribute(swap_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)swap_smem));
   const unsigned srow = div_up(rows, 32);
-  for (int k0 = 0; k0 < n; k0 += kP) {
+  // The next step's panel is updated first and factored on a second stream, by one cluster's
+  // SMs, while the others update the rest: the panel's latency-bound columns would otherwise
+  // leave most of the GPU idle for a third of the time.  The rest waits until the panel has
+  // been copied, so that the cluster (16 SMs of one processing cluster of the chip) is
+  // placed before the update's blocks take their SMs (n = 9,836: LOOKFIG).
+  SideStream side;
+  MSP_TRY(side.create());
+  // The factors of a step's panel (X, D and its digits, the exchanges) on stream f
+  auto factor = [&](int k0, cudaStream_t f) -> int {
     const int kb = std::min(kP, n - k0), m = n - k0;
-    panel_copy_kernel<<<grid_for((size_t)m * kP, 256), 256, 0, s>>>(m, k0, kb, lda, A.p, X.p);
+    panel_copy_kernel<<<grid_for((size_t)m * kP / 2, 256), 256, 0, f>>>(m, k0, kb, act, A.p, X.p);
     MSP_TRY(launch_status());
+    MSP_CUDA_TRY(cudaEventRecord(side.copied, f));
     // the widest sub-panel whose rows fit the registers of one cluster
     constexpr int kLuRows = kMaxCluster * kLuThreads;
     if (m <= kLuRows)
-      MSP_TRY((lu_panel<16, 1>(m, kb, k0, X.p, piv.p, flags, s)));
+      MSP_TRY((lu_panel<16, 1>(m, kb, k0, X.p, piv.p, flags, f)));
     else if (m <= 2 * kLuRows)
-      MSP_TRY((lu_panel<8, 2>(m, kb, k0, X.p, piv.p, flags, s)));
+      MSP_TRY((lu_panel<8, 2>(m, kb, k0, X.p, piv.p, flags, f)));
     else if (m <= 4 * kLuRows)
-      MSP_TRY((lu_panel<4, 4>(m, kb, k0, X.p, piv.p, flags, s)));
+      MSP_TRY((lu_panel<4, 4>(m, kb, k0, X.p, piv.p, flags, f)));
     else if (m <= 16 * kLuRows)
-      MSP_TRY((lu_panel<2, 16>(m, kb, k0, X.p, piv.p, flags, s)));
+      MSP_TRY((lu_panel<2, 16>(m, kb, k0, X.p, piv.p, flags, f)));
     else
       return MSP_ERR_NOMEM;  // two dense copies of such a matrix exceed the device
-    diag_inverse_panel_kernel<<<kP / kDiagWarps + 1, kDiagWarps * kWarp, diag_smem, s>>>(
+    diag_inverse_panel_kernel<<<kP / kDiagWarps + 1, kDiagWarps * kWarp, diag_smem, f>>>(
         k0, kb, X.p, piv.p, D.p, SD.p, ed.p, perm.p, pivots.p);
-    MSP_TRY(launch_status());
-    swap_slice_kernel<<<lda / kColTile, 256, swap_smem, s>>>(lda, k0, kb, A.p, perm.p, ST.p, et.p);
+    return launch_status();
+  };
+  MSP_TRY(factor(0, s));
+  for (int k0 = 0; k0 < n; k0 += kP) {
+    const int kb = std::min(kP, n - k0), kt0 = k0 / kColTile;
+    if (k0 > 0) MSP_CUDA_TRY(cudaStreamWaitEvent(s, side.factored, 0));
+    swap_slice_kernel<<<act, 256, swap_smem, s>>>(act, k0, kb, A.p, perm.p, ST.p, et.p);
     MSP_TRY(launch_status());
     // P = -A_iK D (D for the rows K), then one correction: with the digit products the
     // residual P A_KK + A_iK is nearly exact, so P ends as accurate as its last rounding,
     // however the explicit inverse D of an ill-conditioned block was
     const unsigned pt = (unsigned)std::min(sm_count(), nrt * kKTiles);
-    double* AK = A.p + k0;
-    const char* SK = ST.p + (size_t)(k0 / kColTile) * kTileB;
-    slice_rows_kernel<<<srow, 256, 0, s>>>(lda, k0, k0, k0 + kb, A.p, SA.p, ea.p, Y.p);
+    const char* SK = ST.p + (size_t)kt0 * kTileB;
+    slice_rows_kernel<<<srow, 256, 0, s>>>(act, k0, k0, k0 + kb, A.p, SA.p, ea.p, Y.p);
     MSP_TRY(launch_status());
     slice_gemm_kernel<kFirst><<<pt, kGemmThreads, kGemmSmem, s>>>(
-        lda, k0, kb, nrt, kKTiles, 0, AK, SA.p, ea.p, SD.p, ed.p, D.p, flags);
+        act, kt0, k0, kb, nrt, kKTiles, 0, 0, 0, A.p, SA.p, ea.p, SD.p, ed.p, D.p, flags);
     MSP_TRY(launch_status());
-    slice_rows_kernel<<<srow, 256, 0, s>>>(lda, k0, 0, 0, A.p, SA.p, ea.p, nullptr);
+    slice_rows_kernel<<<srow, 256, 0, s>>>(act, k0, 0, 0, A.p, SA.p, ea.p, nullptr);
     MSP_TRY(launch_status());
     slice_gemm_kernel<kResid><<<pt, kGemmThreads, kGemmSmem, s>>>(
-        kP, k0, kb, nrt, kKTiles, 0, Y.p, SA.p, ea.p, SK, et.p + k0, D.p, flags);
+        kKTiles, 0, k0, kb, nrt, kKTiles, 0, 0, 0, Y.p, SA.p, ea.p, SK, et.p + k0, D.p, flags);
     MSP_TRY(launch_status());
-    slice_rows_kernel<<<srow, 256, 0, s>>>(kP, 0, 0, 0, Y.p, SA.p, ea.p, nullptr);
+    slice_rows_kernel<<<srow, 256, 0, s>>>(kKTiles, 0, 0, 0, Y.p, SA.p, ea.p, nullptr);
     MSP_TRY(launch_status());
     slice_gemm_kernel<kCorrect><<<pt, kGemmThreads, kGemmSmem, s>>>(
-        lda, k0, kb, nrt, kKTiles, 0, AK, SA.p, ea.p, SD.p, ed.p, D.p, flags);
+        act, kt0, k0, kb, nrt, kKTiles, 0, 0, 0, A.p, SA.p, ea.p, SD.p, ed.p, D.p, flags);
     MSP_TRY(launch_status());
-    const int ncu = nct - std::min(nct - k0 / kColTile, kKTiles);
-    if (ncu <= 0) continue;
-    slice_rows_kernel<<<srow, 256, 0, s>>>(lda, k0, 0, 0, A.p, SA.p, ea.p, nullptr);
+    const int nown = std::min(nct - kt0, kKTiles), nnext = std::min(nct - kt0 - nown, kKTiles);
+    if (nct - nown <= 0) continue;
+    slice_rows_kernel<<<srow, 256, 0, s>>>(act, k0, 0, 0, A.p, SA.p, ea.p, nullptr);
     MSP_TRY(launch_status());
-    const long long tiles = (long long)nrt * ncu;
-    slice_gemm_kernel<kUpdate><<<(unsigned)std::min<long long>(sm_count(), tiles), kGemmThreads,
-                                 kGemmSmem, s>>>(lda, k0, kb, nrt, ncu, k0 / kColTile, A.p, SA.p,
-                                                 ea.p, ST.p, et.p, D.p, flags);
-    MSP_TRY(launch_status());
+    auto update = [&](int count, int cbegin, int skip_at, int skip, int blocks) -> int {
+      const long long tiles = (long long)nrt * count;
+      if (tiles <= 0) return MSP_OK;
+      slice_gemm_kernel<kUpdate><<<(unsigned)std::min<long long>(blocks, tiles), kGemmThreads,
+                                   kGemmSmem, s>>>(act, 0, k0, kb, nrt, count, cbegin, skip_at, skip,
+                                                   A.p, SA.p, ea.p, ST.p, et.p, D.p, flags);
+      return launch_status();
+    };
+    MSP_TRY(update(nnext, kt0 + nown, nnext, 0, sm_count()));
+    if (nnext > 0) {
+      MSP_CUDA_TRY(cudaEventRecord(side.ready, s));
+      MSP_CUDA_TRY(cudaStreamWaitEvent(side.stream, side.ready, 0));
+      MSP_TRY(factor(k0 + kP, side.stream));
+      MSP_CUDA_TRY(cudaEventRecord(side.factored, side.stream));
+      MSP_CUDA_TRY(cudaStreamWaitEvent(s, side.copied, 0));
+    }
+    MSP_TRY(update(nct - nown - nnext, 0, kt0, nown + nnext,
+                   nnext > 0 ? std::max(1, sm_count() - kMaxCluster) : sm_count()));
   }
   std::vector<int> hp(n), cols(n);
   DevFlags hf{};
@@ -1107,7 +1198,7 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
   for (int k = n - 1; k >= 0; --k)
     if (hp[k] != k) std::swap(cols[k], cols[hp[k]]);
   MSP_CUDA_TRY(cudaMemcpyAsync(cols_d.p, cols.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
-  unscramble_kernel<<<grid_for((size_t)n * n, 256), 256, 0, s>>>(n, lda, cols_d.p, A.p, out);
+  unscramble_kernel<<<dim3(div_up(n, 32), div_up(n, 32)), 256, 0, s>>>(n, act, cols_d.p, A.p, out);
   MSP_TRY(launch_status());
   MSP_CUDA_TRY(cudaStreamSynchronize(s));  // cols and the temporaries are in use until here
   return MSP_OK;
