@@ -19,9 +19,12 @@
 // side (N = 32 (9 - i)), each into the accumulator columns of its i + j.
 //
 // One SETUP's inverse, before (rank-32 updates on the FP64 pipes, two launches per column)
-// and now: n = 2,048: 45 -> 13 ms, 4,231: 203 -> 36 ms, 5,867: 446 -> 62 ms, 9,836: 1,824 ->
-// 178 ms (21 TFLOP/s of FP64 arithmetic).  Errors against an extended-precision solve are
-// below the previous kernels' (9,836 rows: 7.5e-16 against 1.8e-15).
+// and now: n = 2,048: 45 -> 13 ms, 4,231: 203 -> 30 ms, 5,867: 446 -> 46 ms, 9,836: 1,824 ->
+// 109 ms (17 FP64 TFLOP/s).  Errors against an extended-precision solve are below the
+// previous kernels' (9,836 rows: 7.5e-16 against 1.8e-15).  What bounds it: the panels'
+// columns (3.5 us each, a chain of one cluster exchange, a reciprocal and the rank-1
+// update) up to about 6,000 rows, above that the products, whose epilogue keeps the FP64
+// pipe and the trips to TMEM and memory busy (tensor pipe 25 %).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -60,7 +63,7 @@ inline int launch_status() { return launch_check(__FILE__, __LINE__); }
 // The dense matrices are stored by tiles of 128 rows x 32 columns (row tiles of `nct` column
 // tiles), a tile by pairs of columns, then rows: the 32 rows that a warp of the products'
 // epilogue holds are 512 consecutive bytes.  (With rows of the whole matrix each lane
-// touched its own line: 2.7 times the sectors, n = 9,836 157 -> LAYFIG ms.)
+// touched its own line and the L1 was the busiest unit: n = 9,836 157 -> 126 ms, 5,867 57 -> 47 ms.)
 __device__ __forceinline__ size_t tile_at(int nct, int i, int j) {
   return ((size_t)(i / kRowTile) * nct + j / kColTile) * (kRowTile * kColTile) +
          (size_t)((j % kColTile) / 2) * (2 * kRowTile) + (i % kRowTile) * 2 + (j & 1);
@@ -1043,8 +1046,7 @@ int lu_panel(int m, int kb, int k0, double* X, int* piv, DevFlags* flags, cudaSt
   return MSP_OK;
 }
 
-// A stream of its own for the panels (of high priority, so that a panel's cluster is placed
-// before the update's blocks), joined before it goes
+// A stream of its own for the panels, joined before it goes
 struct SideStream {
   cudaStream_t stream = nullptr;
   cudaEvent_t ready = nullptr, copied = nullptr, factored = nullptr;
@@ -1052,9 +1054,7 @@ struct SideStream {
   SideStream(const SideStream&) = delete;
   SideStream& operator=(const SideStream&) = delete;
   int create() {
-    int least = 0, greatest = 0;
-    MSP_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    MSP_CUDA_TRY(cudaStreamCreateWithPriority(&stream, cudaStreamNonBlocking, greatest));
+    MSP_CUDA_TRY(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
     MSP_CUDA_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
     MSP_CUDA_TRY(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming));
     MSP_CUDA_TRY(cudaEventCreateWithFlags(&factored, cudaEventDisableTiming));
@@ -1114,7 +1114,8 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
   // SMs, while the others update the rest: the panel's latency-bound columns would otherwise
   // leave most of the GPU idle for a third of the time.  The rest waits until the panel has
   // been copied, so that the cluster (16 SMs of one processing cluster of the chip) is
-  // placed before the update's blocks take their SMs (n = 9,836: LOOKFIG).
+  // placed before the update's blocks take their SMs (n = 16,700: 671 -> 503 ms, 4,231: 35 ->
+  // 31 ms; without that wait the cluster found no place and nothing was gained).
   SideStream side;
   MSP_TRY(side.create());
   // The factors of a step's panel (X, D and its digits, the exchanges) on stream f

@@ -34,11 +34,12 @@ int launch_bsr_spmv_perm(int b, int nb, const int* rp, const int* ci, const doub
                          const int* perm, const double* x, double* y, cudaStream_t s,
                          LongRows lr);
 // rP[i] = omega_i^T (g_i - (A w)_i)   (omega == nullptr: first unknown only); r != nullptr
-// also receives g - A w
+// also receives g - A w.  after_n (with r): the pressure slots of w are zero (stage N)
 template <typename T>
-int launch_bsr_restrict_p(int b, int nb, const int* rp, const int* ci, const T* v,
-                          const T* w, const T* g, const T* omega, T* rP, T* r, cudaStream_t s,
-                          const unsigned char* rmask = nullptr, LongRows lr = LongRows());
+int launch_bsr_restrict_p(int b, int nb, const int* rp, const int* ci, const T* v, const T* w,
+                          const T* g, const T* omega, T* rP, T* r, bool after_n,
+                          cudaStream_t s, const unsigned char* rmask = nullptr,
+                          LongRows lr = LongRows());
 // r_i <- r_i - sum_j A_ij[:, 0] e_j and w_i[0] += e_i (r, w: nb*b values; c0: column 0 of
 // every block, nnzb*b values; e: one value per block row)
 template <typename T>
@@ -95,13 +96,14 @@ int launch_ell_gs_colour(int K, int r0, int r1, const int* ell_ci, const T* ell_
                          const int* dpos, const T* rdiag, const T* b, T* x, bool lower_only,
                          cudaStream_t s, const unsigned char* rmask = nullptr, bool pdl = false,
                          int tpr = 0);
-// the same restriction over the ELL copy of the level (diag: a_ii of every row)
+// the same restriction over the ELL copy of the level (diag: a_ii of every row); upper: x is
+// the result of one forward colour sweep from zero
 template <typename T>
 int launch_ell_residual_restrict(int K, int nc, const int* mptr, const int* members,
                                  const int* ell_ci, const T* ell_v, const int* meta,
                                  const T* diag, const int* rp, const int* ci, const T* v,
-                                 const T* b, const T* x, T* bc, cudaStream_t s,
-                                 const unsigned char* cmask = nullptr, int tpr = 0);
+                                 const int* dpos, const T* b, const T* x, T* bc, cudaStream_t s,
+                                 const unsigned char* cmask, int tpr, bool upper);
 int ell_default_tpr(int K);
 bool ell_tpr_ok(int K, int tpr);
 // PJAC-NO and PGS-NO sweeps in storage order (x0: the values at the start of the sweep,

@@ -1036,6 +1036,13 @@ PView<float> view32(msp_handle h) {
   return p;
 }
 
+// Whether the residual restriction of a level of n rows reads only the entries right of the
+// diagonal (after one forward colour sweep from zero the others cancel): on levels bound
+// by bandwidth.
+bool restrict_upper(msp_handle h, int n) {
+  return h->cfg.smoother == MSP_SMOOTHER_PGS_MC && h->cfg.pre_sweeps == 1 && n > 262144;
+}
+
 // algorithmic bytes of one colour sweep launch over rows [r0, r1) reading `entries`
 // nonzeros of `eb` bytes each (value + column index) plus `rowb` bytes per row
 // The tile autotuner (msp_config.autotune): for every AMG level swept over its ELL copy,
@@ -1097,8 +1104,9 @@ int autotune_levels_t(msp_handle h, const PView<T>& P, cudaStream_t s) {
       st = time_it([&]() -> int {
         return launch_ell_residual_restrict<T>(L.ell_k, L.nc, L.mptr.p, L.members.p, L.ell_ci.p,
                                                P.lev[l], L.ell_meta.p, P.led[l], L.A.rp.p,
-                                               L.A.ci.p, P.lv[l], P.lb[l], P.lx[l],
-                                               P.lb[l + 1], s, nullptr, tpr);
+                                               L.A.ci.p, P.lv[l], L.dpos.p, P.lb[l], P.lx[l],
+                                               P.lb[l + 1], s, nullptr, tpr,
+                                               restrict_upper(h, n));
       }, &t);
       if (st != MSP_OK) break;
       if (t < t_rr) {
@@ -1269,8 +1277,9 @@ int vcycle(msp_handle h, const PView<T>& P, int l, cudaStream_t s) {
       Probe pr(level_site("amg_residual_restrict_l", l), bytes, s);
       MSP_TRY(launch_ell_residual_restrict<T>(L.ell_k, L.nc, L.mptr.p, L.members.p, L.ell_ci.p,
                                               P.lev[l], L.ell_meta.p, P.led[l], L.A.rp.p,
-                                              L.A.ci.p, P.lv[l], P.lb[l], P.lx[l], P.lb[l + 1],
-                                              s, P.lm[l + 1], L.rr_tpr));
+                                              L.A.ci.p, P.lv[l], L.dpos.p, P.lb[l], P.lx[l],
+                                              P.lb[l + 1], s, P.lm[l + 1], L.rr_tpr,
+                                              restrict_upper(h, n)));
     } else {
       Probe pr(level_site("amg_residual_restrict_csr_l", l), bytes, s);
       MSP_TRY(launch_csr_residual_restrict<T>(L.nc, L.mptr.p, L.members.p, L.A.rp.p,
@@ -1357,7 +1366,7 @@ int stage_P(msp_handle h, const PView<T>& P, const T* g, T* w, T* r, cudaStream_
     Probe pr("stageP_residual_restrict", bsr_bytes(h, sT, r ? 3 : 2) + (double)h->nb * sT, s,
              1, sT == 8 ? 2.0 * (bsr_fmas(h) + (double)h->nb * b) : 0.0);
     MSP_TRY(launch_bsr_restrict_p<T>(h->b, h->nb, h->rp.p, h->ci.p, P.vals, w, g, P.omega,
-                                     P.lb[0], r, s, P.m0, long_rows(h, 0, h->nb)));
+                                     P.lb[0], r, true, s, P.m0, long_rows(h, 0, h->nb)));
   }
   MSP_TRY(vcycle<T>(h, P, 0, s));
   if (!r) {

@@ -75,11 +75,11 @@ __device__ __forceinline__ T fma_row(const T (&a)[B], const T (&x)[B], T acc) {
   return acc;
 }
 
-// acc - a . x
-template <int B, typename T>
+// acc - a . x over the columns from C0 on
+template <int B, int C0 = 0, typename T>
 __device__ __forceinline__ T fnma_row(const T (&a)[B], const T (&x)[B], T acc) {
 #pragma unroll
-  for (int c = 0; c < B; ++c) acc = fma(-a[c], x[c], acc);
+  for (int c = C0; c < B; ++c) acc = fma(-a[c], x[c], acc);
   return acc;
 }
 
@@ -334,8 +334,12 @@ __global__ void __launch_bounds__(kThreads) bsr_spmv_kernel(int nb, const int* _
 
 // ----------------------------------------------------------------------------------
 // rP[i] = omega_i^T (g_i - (A w)_i); with WR the residual g - A w is also stored in r
+// AFTERN: w comes from stage N, so its pressure slots are zero and column 0 of the blocks is
+// not multiplied (the FP64 FMAs bound the kernel: 1.12M x 4 242 -> 198 us, 132k x 4 38 ->
+// 33 us).  The concentration rows of the last
+// colour are not zero in general: the matrix may be newer than the preconditioner.
 // ----------------------------------------------------------------------------------
-template <int B, typename T, bool WR>
+template <int B, typename T, bool WR, bool AFTERN>
 __global__ void __launch_bounds__(kThreads) bsr_restrict_p_kernel(
     int nb, const int* __restrict__ rp, const int* __restrict__ ci, const T* __restrict__ v,
     const T* __restrict__ w, const T* __restrict__ g, const T* __restrict__ omega,
@@ -358,7 +362,7 @@ __global__ void __launch_bounds__(kThreads) bsr_restrict_p_kernel(
     for (int k = 1; k < B; ++k) res += __shfl_sync(0xffffffffu, term, k);
     if (l == 0) rP[i] = res;
   }
-  constexpr int GP = Gp<B>::v;
+  constexpr int GP = Gp<B>::v, kFirst = AFTERN ? 1 : 0;  // first column multiplied
   const int lane = threadIdx.x % GP;
   const int gpb = blockDim.x / GP;
   // the loop bound depends on the block only, so every lane reaches the group shuffle
@@ -380,15 +384,15 @@ __global__ void __launch_bounds__(kThreads) bsr_restrict_p_kernel(
         load_row<B>(v + ((size_t)(p + 1) * B + lane) * B, a1);
         load_row<B>(w + (size_t)j0 * B, x0);
         load_row<B>(w + (size_t)j1 * B, x1);
-        acc = fnma_row<B>(a0, x0, acc);
-        acc = fnma_row<B>(a1, x1, acc);
+        acc = fnma_row<B, kFirst>(a0, x0, acc);
+        acc = fnma_row<B, kFirst>(a1, x1, acc);
       }
       if (p < p1) {
         const int j0 = __ldg(ci + p);
         T a0[B], x0[B];
         load_row<B>(v + ((size_t)p * B + lane) * B, a0);
         load_row<B>(w + (size_t)j0 * B, x0);
-        acc = fnma_row<B>(a0, x0, acc);
+        acc = fnma_row<B, kFirst>(a0, x0, acc);
       }
       if (WR) r[(size_t)i * B + lane] = acc;
       res = omega ? acc * omega[(size_t)i * B + lane] : (lane == 0 ? acc : T(0));
@@ -809,13 +813,18 @@ __global__ void __launch_bounds__(kThreads) ell_gs_colour_kernel(
 // per member and S slots per lane, so the member list, the entries and the gather of x
 // are the only dependent trips to memory.  Rows longer than K (meta < 0) walk their CSR
 // row (diagonal included) instead of the slots and the diagonal term.
-template <typename T, int K, int TPR>
+// UPPER (after one forward sweep from zero): a row was solved with the values of the earlier
+// colours and zeros for the later ones, so b_i - (A x)_i is minus its entries right of the
+// diagonal times x, and only those are read, once meta is there.  For levels bound by
+// bandwidth (1.12M rows: 57.6 -> 45.8 us); on small ones the further trip to memory costs more
+// (132k-row application 458 against 476 us with it everywhere).
+template <typename T, int K, int TPR, bool UPPER>
 __global__ void __launch_bounds__(kThreads) ell_residual_restrict_kernel(
     int nc, const int* __restrict__ mptr, const int* __restrict__ members,
     const int* __restrict__ ell_ci, const T* __restrict__ ell_v, const int* __restrict__ meta,
     const T* __restrict__ diag, const int* __restrict__ rp, const int* __restrict__ ci,
-    const T* __restrict__ v, const T* __restrict__ b, const T* __restrict__ x,
-    T* __restrict__ bc, const unsigned char* __restrict__ cmask) {
+    const T* __restrict__ v, const int* __restrict__ dpos, const T* __restrict__ b,
+    const T* __restrict__ x, T* __restrict__ bc, const unsigned char* __restrict__ cmask) {
   constexpr int kMembers = 4, G = kMembers * TPR, S = (K + TPR - 1) / TPR;
   const int lane = threadIdx.x % G;
   const int ms = lane / TPR, t = lane % TPR;
@@ -831,9 +840,34 @@ __global__ void __launch_bounds__(kThreads) ell_residual_restrict_kernel(
       for (int mb = m0 + ms; mb < m1; mb += kMembers) {
         const int i = __ldg(members + mb);
         const int m = __ldg(meta + i);
-        if (t == 0) total += __ldg(b + i);
         int j[S];
         T a[S], xj[S];
+        if constexpr (UPPER) {
+          const int lo = m >> 16, hi = m & 0xffff;  // m < 0: taken below
+#pragma unroll
+          for (int q = 0; q < S; ++q) {
+            const int k = t + q * TPR;
+            const bool need = m >= 0 && k >= lo && k < hi;
+            j[q] = need ? __ldg(ell_ci + (size_t)i * K + k) : i;
+            a[q] = need ? __ldg(ell_v + (size_t)i * K + k) : T(0);
+          }
+#pragma unroll
+          for (int q = 0; q < S; ++q) {
+            const int k = t + q * TPR;
+            xj[q] = m >= 0 && k >= lo && k < hi ? __ldg(x + j[q]) : T(0);
+          }
+          if (m >= 0) {
+#pragma unroll
+            for (int q = 0; q < S; ++q)
+              if (t + q * TPR >= lo) total = fma(-a[q], xj[q], total);
+          } else {
+            const int p1 = __ldg(rp + i + 1);
+            for (int p = __ldg(dpos + i) + 1 + t; p < p1; p += TPR)
+              total = fma(-__ldg(v + p), __ldg(x + __ldg(ci + p)), total);
+          }
+          continue;
+        }
+        if (t == 0) total += __ldg(b + i);
 #pragma unroll
         for (int q = 0; q < S; ++q) {
           const int k = t + q * TPR;
@@ -1753,16 +1787,19 @@ int launch_bsr_spmv_perm(int b, int nb, const int* rp, const int* ci, const doub
 
 template <typename T>
 int launch_bsr_restrict_p(int b, int nb, const int* rp, const int* ci, const T* v, const T* w,
-                          const T* g, const T* omega, T* rP, T* r, cudaStream_t s,
-                          const unsigned char* rmask, LongRows lr) {
+                          const T* g, const T* omega, T* rP, T* r, bool after_n,
+                          cudaStream_t s, const unsigned char* rmask, LongRows lr) {
   if (nb <= 0) return MSP_OK;
   MSP_B_SWITCH(b, {
     const unsigned grid = with_long_rows(grid_groups(nb, Gp<B_>::v), lr.n);
-    if (r)
-      bsr_restrict_p_kernel<B_, T, true><<<grid, kThreads, 0, s>>>(
+    if (r && after_n)
+      bsr_restrict_p_kernel<B_, T, true, true><<<grid, kThreads, 0, s>>>(
+          nb, rp, ci, v, w, g, omega, rP, r, rmask, lr.rows, lr.n, lr.thr);
+    else if (r)
+      bsr_restrict_p_kernel<B_, T, true, false><<<grid, kThreads, 0, s>>>(
           nb, rp, ci, v, w, g, omega, rP, r, rmask, lr.rows, lr.n, lr.thr);
     else
-      bsr_restrict_p_kernel<B_, T, false><<<grid, kThreads, 0, s>>>(
+      bsr_restrict_p_kernel<B_, T, false, false><<<grid, kThreads, 0, s>>>(
           nb, rp, ci, v, w, g, omega, rP, r, rmask, lr.rows, lr.n, lr.thr);
   });
   return launch_status();
@@ -2008,17 +2045,20 @@ template <typename T>
 int launch_ell_residual_restrict(int K, int nc, const int* mptr, const int* members,
                                  const int* ell_ci, const T* ell_v, const int* meta,
                                  const T* diag, const int* rp, const int* ci, const T* v,
-                                 const T* b, const T* x, T* bc, cudaStream_t s,
-                                 const unsigned char* cmask, int tpr) {
+                                 const int* dpos, const T* b, const T* x, T* bc, cudaStream_t s,
+                                 const unsigned char* cmask, int tpr, bool upper) {
   if (nc <= 0) return MSP_OK;
   if (tpr == 0) tpr = ell_default_tpr(K);
   if (!ell_tpr_ok(K, tpr)) return MSP_ERR_ARG;
   switch (K * 16 + tpr) {
 #define MSP_ELLR_CASE(KK, TT)                                                               \
-  case KK * 16 + TT:                                                                        \
-    ell_residual_restrict_kernel<T, KK, TT><<<grid_groups(nc, 4 * TT), kThreads, 0, s>>>(   \
-        nc, mptr, members, ell_ci, ell_v, meta, diag, rp, ci, v, b, x, bc, cmask);         \
-    break;
+  case KK * 16 + TT: {                                                                      \
+    auto* kern = upper ? ell_residual_restrict_kernel<T, KK, TT, true>                      \
+                       : ell_residual_restrict_kernel<T, KK, TT, false>;                    \
+    kern<<<grid_groups(nc, 4 * TT), kThreads, 0, s>>>(nc, mptr, members, ell_ci, ell_v,     \
+                                                      meta, diag, rp, ci, v, dpos, b, x,    \
+                                                      bc, cmask);                           \
+  } break;
     MSP_ELLR_CASE(8, 2)
     MSP_ELLR_CASE(8, 4)
     MSP_ELLR_CASE(8, 8)
@@ -2296,8 +2336,8 @@ int launch_scatter_blocks(int nb, int b, const int* perm, const double* in, doub
                                   const T*, T*, bool, cudaStream_t, const unsigned char*,   \
                                   LongRows);                                                \
   template int launch_bsr_restrict_p<T>(int, int, const int*, const int*, const T*,         \
-                                        const T*, const T*, const T*, T*, T*, cudaStream_t, \
-                                        const unsigned char*, LongRows);                    \
+                                        const T*, const T*, const T*, T*, T*, bool,         \
+                                        cudaStream_t, const unsigned char*, LongRows); \
   template int launch_bsr_col0_update<T>(int, int, const int*, const int*, const T*,        \
                                          const T*, T*, T*, cudaStream_t, const unsigned char*, \
                                          LongRows);                                          \
@@ -2323,8 +2363,9 @@ int launch_scatter_blocks(int nb, int b, const int* perm, const double* in, doub
                                        const unsigned char*, bool, int);                  \
   template int launch_ell_residual_restrict<T>(int, int, const int*, const int*, const int*, \
                                                const T*, const int*, const T*, const int*,  \
-                                               const int*, const T*, const T*, const T*, T*, \
-                                               cudaStream_t, const unsigned char*, int);                               \
+                                               const int*, const T*, const int*, const T*,  \
+                                               const T*, T*, cudaStream_t,                  \
+                                               const unsigned char*, int, bool);            \
   template int launch_jacobi_sweep<T>(int, const int*, const int*, const T*, const int*,    \
                                       const T*, const T*, const T*, T*, cudaStream_t);      \
   template int launch_pgs_no_sweep<T>(int, const int*, const int*, const T*, const int*,    \
