@@ -20,7 +20,7 @@
 //
 // One SETUP's inverse, before (rank-32 updates on the FP64 pipes, two launches per column)
 // and now: n = 2,048: 45 -> 13 ms, 4,231: 203 -> 30 ms, 5,867: 446 -> 46 ms, 9,836: 1,824 ->
-// 109 ms (17 FP64 TFLOP/s).  Errors against an extended-precision solve are below the
+// 109 to 135 ms (14 to 17 FP64 TFLOP/s, as the panels' clusters find their place).  Errors against an extended-precision solve are below the
 // previous kernels' (9,836 rows: 7.5e-16 against 1.8e-15).  What bounds it: the panels'
 // columns (3.5 us each, a chain of one cluster exchange, a reciprocal and the rank-1
 // update) up to about 6,000 rows, above that the products, whose epilogue keeps the FP64
