@@ -98,8 +98,10 @@ __device__ __forceinline__ T group_sum(T v) {
 // q0 + t / R, q0 + t / R + NB, ...), the same few registers per thread as the lane-group
 // kernels; thread r < R returns S_r, the partial sums combined through shared memory in
 // a fixed order.  Every thread of the block calls it (it synchronises the block).  x rows
-// are never written by the launch.
-template <int R, int C, typename T>
+// are never written by the launch.  DEP: the launch is a programmatic dependent and x may
+// still have been written after it started, so x is read from L2 instead of through the
+// read-only path.
+template <int R, int C, bool DEP = false, typename T>
 __device__ __forceinline__ T block_row_sum(int q0, int q1, int skip, const int* __restrict__ ci,
                                            const T* __restrict__ vals, const T* x, int xs,
                                            int xo, const int* __restrict__ perm = nullptr) {
@@ -117,7 +119,8 @@ __device__ __forceinline__ T block_row_sum(int q0, int q1, int skip, const int* 
       const T* xr = x + (size_t)(perm ? __ldg(perm + j) : j) * xs + xo;
       const T* a = vals + ((size_t)q * R + r) * C;
 #pragma unroll
-      for (int c = 0; c < C; ++c) part = fma(__ldg(a + c), __ldg(xr + c), part);
+      for (int c = 0; c < C; ++c)
+        part = fma(__ldg(a + c), DEP ? __ldcg(xr + c) : __ldg(xr + c), part);
     }
   }
   part_s[t] = part;
@@ -483,8 +486,8 @@ __global__ void __launch_bounds__(kThreads) bgs_colour_kernel(
       const int i = lrows[q];
       if (rmask && !rmask[i]) continue;
       const int pd = __ldg(dpos + i);
-      const T sl = block_row_sum<BN, BN>(__ldg(rp + i), lower_only ? pd : __ldg(rp + i + 1), pd,
-                                        ci, aN, w, B, 1);
+      const T sl = block_row_sum<BN, BN, PDL>(
+          __ldg(rp + i), lower_only ? pd : __ldg(rp + i + 1), pd, ci, aN, w, B, 1);
       if (threadIdx.x >= kWarp) continue;  // the row's outputs are warp 0's
       const int l = threadIdx.x;
       if (l < BN) w[(size_t)i * B + 1 + l] = __ldcg(y + (size_t)i * BN + l) - sl;
