@@ -237,9 +237,9 @@ __global__ void __launch_bounds__(kThreads) bilu_fwd_long_colour_kernel(
     return;
   }
   const int l = threadIdx.x;
-  const T rl = l < B ? __ldg(r + (size_t)i * B + l) : T(0);
   const T sl = long_colour_row_sum<B, B, T, PDL>(__ldg(rp + i), __ldg(dpos + i), -1, ci, lu, y, B, 0);
-  if (l < B) y[(size_t)i * B + l] = rl - sl;
+  // r after the wait: the kernel that wrote it comes right before the first colour
+  if (l < B) y[(size_t)i * B + l] = __ldcg(r + (size_t)i * B + l) - sl;
 }
 
 // BILU(0) backward over a colour of long rows only: x_i = U_ii^-1 (y_i - sum_{j>i} U_ij x_j)
