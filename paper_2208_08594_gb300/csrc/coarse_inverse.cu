@@ -1,5 +1,7 @@
-// Dense FP64 inverse of the coarsest AMG matrix (Section 5: a direct solver), by blocked
-// in-place Gauss-Jordan with partial pivoting.  One step takes the kP = 96 columns K:
+// Dense FP64 inverse of the coarsest AMG matrix (Section 5: a direct solver).  The matrix is
+// scaled by powers of two per row and column (exact; undone at the end), inverted by blocked
+// in-place Gauss-Jordan with partial pivoting, and the inverse corrected once.  One step of the
+// elimination takes the kP = 96 columns K:
 //   1. LU with partial pivoting of the rows k0..n-1 of a copy of those columns, in
 //      sub-panels of W columns by one thread-block cluster (lu_panel_kernel) with rank-W
 //      updates of the rest of the copy in between (lu_update_kernel);
@@ -8,15 +10,29 @@
 //   3. A_iK <- P_iK = -A_iK D for the rows outside K, A_KK <- D, and with T = A_K,: before
 //      the step, A_ij += P_iK T_j outside K and A_Kj = D T_j (slice_gemm_kernel).
 // Step 3 is 2 n^3 flops in all.  The FP64 pipes do 1.25 TFLOP/s on this part, so it runs on
-// the fifth-generation tensor cores instead, without losing precision: every FP64 operand
-// is scaled by a power of two per row of P (per column of T) and written as eight signed
-// radix-256 digits, integers that bf16 holds exactly.  The product of two digits is at most
-// 2^14, and the sum over 96 terms and the up to eight digit pairs (i, j) with the same i + j
-// at most 8 * 96 * 2^14 < 2^24, so every FP32 accumulator holds an exact integer.  The 36
-// pairs with i + j <= 9 are kept (seven digits lost accuracy where a row's entries differ
-// widely); an epilogue adds the eight sums in integer arithmetic and rounds when it adds
-// them to C.  Every instruction multiplies digit i of P by the digits 1..9-i of T side by
-// side (N = 32 (9 - i)), each into the accumulator columns of its i + j.
+// the fifth-generation tensor cores instead, by the error-free splitting of Ozaki, Ogita, Oishi
+// and Rump (Numer. Algorithms 59, 2012): every FP64 operand is scaled by a power of two per row
+// of P (per column of T) and written as eight signed radix-256 digits, integers that bf16 holds
+// exactly.  The product of two digits is at most 2^14, and the sum over 96 terms and the up to
+// eight digit pairs (i, j) with the same i + j at most 8 * 96 * 2^14 < 2^24, so every FP32
+// accumulator holds an exact integer.  The 36 pairs with i + j <= 9 are kept (seven digits lost
+// accuracy where a row's entries differ widely); an epilogue adds the eight sums in integer
+// arithmetic and rounds when it adds them to C.  Every instruction multiplies digit i of P by
+// the digits 1..9-i of T side by side (N = 32 (9 - i)), each into the accumulator columns of its
+// i + j.
+//
+// Such a product is exact to about 2^-56 of the row's times the column's largest operand: as an
+// FP64 product in norm, but its small entries lose what FP64 products of small operands keep,
+// and where rows of A are in other units than the rest that reaches the large entries (four
+// rows times 1e10: 2e-9 of the largest entry; FP64 elimination 5e-15).  Hence the scaling, and
+// after the elimination one step X += X (I - B X): the residual in FP64 from the sparse matrix B,
+// the product in six digits of the already small term (four left entries of 1e-14 of the largest
+// with fewer correct digits than FP64 elimination where the permeability spans e^(4N)).
+// Errors of the algorithm against an extended-precision inverse, with FP64 elimination in
+// parentheses, as a fraction of the largest entry and of the entry itself: coarsest level of 742
+// rows 1.7e-16 (8.2e-16) and 3.5e-13 (9.4e-13); permeabilities e^(4N) 7.5e-15 (1.1e-14) and
+// 5.2e-13 (2.4e-11); rows times 10^U[-9,9] 9e-17 (1e-11) and 7e-16 (7e-6); elimination with an
+// exchange in every column, 1,000 rows, 1.1e-14 (1.5e-13) and 6e-10 (1.6e-8).
 //
 // One SETUP's inverse, before (rank-32 updates on the FP64 pipes, two launches per column)
 // and now: n = 2,048: 45 -> 13 ms, 4,231: 203 -> 30 ms, 5,867: 446 -> 46 ms, 9,836: 1,824 ->
@@ -40,22 +56,30 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kP = 96;         // columns of a Gauss-Jordan step
-constexpr int kDigits = 8;     // radix-256 digits of an operand
 constexpr int kRowTile = 128;  // rows of a product tile (one MMA's M)
 constexpr int kColTile = 32;   // columns of a product tile
 constexpr int kKTiles = kP / kColTile;
 constexpr int kChunk = 16;     // columns of K per copy (one MMA's K)
-constexpr int kChunks = kP / kChunk;
 constexpr int kStages = 4;     // chunk buffers of a column tile's digits
-constexpr int kGroups = kDigits;  // sums of digit pairs with equal i + j = 2..9
-// bytes of one K chunk of a row tile's / column tile's digits (bf16, core matrices of 8
-// rows x 16 bytes; kc: 16-byte groups along K)
+// A product's operands in ND radix-256 digits over kK columns: eight digits and 96 columns in
+// the elimination, six and 128 in the correction (the same bytes, and the same bound
+// ND kK 2^14 < 2^24 on the sums).  Bytes of one K chunk of a row tile's / column tile's
+// digits (bf16, core matrices of 8 rows x 16 bytes).
 constexpr int kSliceA = kRowTile * kChunk * 2;            // one digit of a row tile
-constexpr int kChunkA = kDigits * kSliceA;                // 32,768
-constexpr int kTileA = kChunks * kChunkA;                 // 196,608
-constexpr int kRowsB = kDigits * kColTile;                // digits side by side
-constexpr int kChunkB = kRowsB * kChunk * 2;              // 8,192
-constexpr int kTileB = kChunks * kChunkB;                 // 49,152
+template <int ND>
+struct Geo {
+  static constexpr int kK = 8 * kP / ND;                  // columns of K per product
+  static constexpr int kChunks = kK / kChunk;
+  static constexpr int kChunkA = ND * kSliceA;            // 32,768 or 24,576
+  static constexpr int kRowsB = ND * kColTile;            // digits side by side
+  static constexpr int kChunkB = kRowsB * kChunk * 2;     // 8,192 or 6,144
+  static constexpr int kDigitB = (kColTile / 8) * 128;    // one digit of a column tile's chunk
+};
+constexpr int kTileA = Geo<8>::kChunks * Geo<8>::kChunkA;  // 196,608
+constexpr int kTileB = Geo<8>::kChunks * Geo<8>::kChunkB;  // 49,152
+constexpr int kCorrDigits = 6;
+using CorrGeo = Geo<kCorrDigits>;
+static_assert(CorrGeo::kChunks * CorrGeo::kChunkA == kTileA && CorrGeo::kChunks * CorrGeo::kChunkB == kTileB);
 constexpr int kZeroExp = -4000;                           // exponent of an all-zero row
 
 inline int launch_status() { return launch_check(__FILE__, __LINE__); }
@@ -98,15 +122,19 @@ __device__ __forceinline__ unsigned bf16_of_int(int d) {  // exact for |d| <= 25
   return __float_as_uint((float)d) >> 16;
 }
 
-// the digits of eight consecutive operands along K, packed eight bf16 per digit:
+// the ND leading digits of eight consecutive operands along K, packed eight bf16 per digit:
 // digit s (0 = most significant) to dst + s * stride
+template <int ND>
 __device__ __forceinline__ void store_digits8(const double (&x)[8], int e, char* dst,
                                               size_t stride) {
   long long v[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) v[q] = scaled_int(x[q], e);
+  for (int q = 0; q < 8; ++q) {
+    v[q] = scaled_int(x[q], e);
+    if (ND < 8) v[q] = ((v[q] >> (63 - 8 * ND)) + 1) >> 1;  // rounded to the digits kept
+  }
 #pragma unroll
-  for (int s = kDigits - 1; s >= 0; --s) {
+  for (int s = ND - 1; s >= 0; --s) {
     unsigned w[4];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -125,6 +153,20 @@ __device__ __forceinline__ void store_digits8(const double (&x)[8], int e, char*
     }
     *reinterpret_cast<uint4*>(dst + (size_t)s * stride) = make_uint4(w[0], w[1], w[2], w[3]);
   }
+}
+
+// digit 0 of row i, 16-byte group kcg of K, in the row tiles' images
+template <int ND>
+__device__ __forceinline__ char* digit_a(char* S, int i, int kcg) {
+  const int tr = i % kRowTile;
+  return S + (size_t)(i / kRowTile) * kTileA + (size_t)(kcg / 2) * Geo<ND>::kChunkA +
+         (kcg % 2) * (kRowTile / 8) * 128 + (tr / 8) * 128 + (tr % 8) * 16;
+}
+// digit 0 of column c (of a tile of 32), 16-byte group kcg of K, in a column tile's image
+template <int ND>
+__device__ __forceinline__ char* digit_b(char* tile, int c, int kcg) {
+  return tile + (size_t)(kcg / 2) * Geo<ND>::kChunkB + (kcg % 2) * (Geo<ND>::kRowsB / 8) * 128 +
+         (c / 8) * 128 + (c % 8) * 16;
 }
 
 // Digits of the rows of a tile of 32 rows of A[:, k0..k0+96) (A padded: whole tiles exist),
@@ -171,25 +213,14 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(int nct, int k0, int z0
     }
   }
   __syncthreads();
-  char* tile = S + (size_t)(r0 / kRowTile) * kTileA;
   for (int t = threadIdx.x; t < 32 * (kP / 8); t += 256) {
     const int r = t % 32, kcg = t / 32;
     double x[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) x[q] = sh[r][kcg * 8 + q];
-    const int tr = (r0 + r) % kRowTile;
-    char* dst = tile + (size_t)(kcg / 2) * kChunkA + (kcg % 2) * (kRowTile / 8) * 128 +
-                (tr / 8) * 128 + (tr % 8) * 16;
-    store_digits8(x, se[r], dst, kSliceA);
+    store_digits8<8>(x, se[r], digit_a<8>(S, r0 + r, kcg), kSliceA);
   }
 }
-
-// digit s of column c (of a tile of 32), 16-byte group kcg of K, in a column tile's image
-__device__ __forceinline__ char* digit_b(char* tile, int c, int kcg) {
-  return tile + (size_t)(kcg / 2) * kChunkB + (kcg % 2) * (kRowsB / 8) * 128 + (c / 8) * 128 +
-         (c % 8) * 16;
-}
-constexpr int kDigitStrideB = (kColTile / 8) * 128;
 
 // The panel's row exchanges on a tile of 32 columns of A, and the digits of the exchanged
 // rows K (T, for the tiles of K the block A_KK).  perm[0] = number of rows that change, then pairs
@@ -245,7 +276,7 @@ __global__ void __launch_bounds__(256) swap_slice_kernel(int nct, int k0, int kb
     double x[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) x[q] = sh[kcg * 8 + q][c];
-    store_digits8(x, se[c], digit_b(tile, c, kcg), kDigitStrideB);
+    store_digits8<8>(x, se[c], digit_b<8>(tile, c, kcg), Geo<8>::kDigitB);
   }
 }
 
@@ -654,14 +685,14 @@ __global__ void __launch_bounds__(kDiagWarps * kWarp) diag_inverse_panel_kernel(
   for (int a = 0; a < 3; ++a) {
     const int q = lane + 32 * a;
     long long v = scaled_int(y[a], e);
-    char* dst = digit_b(tile, j % kColTile, q / 8) + (q % 8) * 2;
-    for (int s = kDigits - 1; s >= 0; --s) {
+    char* dst = digit_b<8>(tile, j % kColTile, q / 8) + (q % 8) * 2;
+    for (int s = 7; s >= 0; --s) {
       int d = (int)v;
       if (s > 0) {
         d = (int)(((unsigned)v + 128u) & 255u) - 128;
         v = (v - d) >> 8;
       }
-      *reinterpret_cast<unsigned short*>(dst + (size_t)s * kDigitStrideB) =
+      *reinterpret_cast<unsigned short*>(dst + (size_t)s * Geo<8>::kDigitB) =
           (unsigned short)bf16_of_int(d);
     }
   }
@@ -738,9 +769,23 @@ __device__ __forceinline__ void tmem_ld8(unsigned addr, unsigned (&r)[8]) {
       : "r"(addr));
 }
 
-// c + sign 2^e sum_m S_m 2^(8 (9 - m)), m = 2..9, S_m exact integers below 2^24
-__device__ __forceinline__ double add_digits(const float (&S)[kGroups], int e, double sign,
-                                             double c) {
+// c + 2^(e + 16) sum_m S_m 2^(8 (5 - m)), m = 0..5, S_m exact integers below 2^24 (as below,
+// with two words of three digits)
+__device__ __forceinline__ double add_digits(const float (&S)[6], int e, double, double c) {
+  const int s0 = __float2int_rn(S[0]), s1 = __float2int_rn(S[1]), s2 = __float2int_rn(S[2]);
+  const int s3 = __float2int_rn(S[3]), s4 = __float2int_rn(S[4]), s5 = __float2int_rn(S[5]);
+  const long long hi = (long long)s0 * 65536 + ((long long)s1 * 256 + s2);
+  const long long lo = (long long)s3 * 65536 + ((long long)s4 * 256 + s5);
+  // M = 1.5 * 2^52 = 1.5 * 2^28 * 2^24
+  const double dh =
+      __longlong_as_double(0x4338000000000000LL + (hi - 402653184)) - 6755399441055744.0;
+  const double dl = __longlong_as_double(0x4338000000000000LL + lo);
+  const int be = min(max(e + 1039, 0), 0x7ff), bh = min(max(e + 1063, 0), 0x7ff);
+  return fma(dl, __longlong_as_double((long long)be << 52),
+             fma(dh, __longlong_as_double((long long)bh << 52), c));
+}
+// c + sign 2^e sum_m S_m 2^(8 (7 - m)), m = 0..7, S_m exact integers below 2^24
+__device__ __forceinline__ double add_digits(const float (&S)[8], int e, double sign, double c) {
   // two exact 64-bit integers, |lo| < 2^49 and |hi| < 2^49; the sum is hi 2^32 + lo
   const int s2 = __float2int_rn(S[0]), s3 = __float2int_rn(S[1]), s4 = __float2int_rn(S[2]);
   const int s5 = __float2int_rn(S[3]), s6 = __float2int_rn(S[4]), s7 = __float2int_rn(S[5]);
@@ -767,7 +812,7 @@ __device__ __forceinline__ double add_digits(const float (&S)[kGroups], int e, d
 //   kUpdate: C = A, the nct column tiles from cbegin, without the kskip tiles from kt0 on (the
 //            columns K and those done by another launch): C += V, or C = V for the rows K;
 //   kFirst:  C = the columns K: C = -V, or D for the rows K;
-//   kResid:  C += V;  kCorrect: C -= V (both on 96 columns).
+//   kResid:  C += V;  kCorrect: C -= V (both on 96 columns; with ND = 6, kResid on all of them).
 enum Product { kUpdate, kFirst, kResid, kCorrect };
 // Persistent blocks, each a contiguous run of tiles in row-major tile order; the digits of a
 // row tile (192 KB) stay in shared memory while the column tiles' digits (48 KB) stream
@@ -777,13 +822,14 @@ enum Product { kUpdate, kFirst, kResid, kCorrect };
 constexpr int kEpiWarps = 16;
 constexpr int kGemmThreads = (kEpiWarps + 2) * kWarp;
 constexpr int kEpiCols = kColTile / (kEpiWarps / 4);  // columns of a tile per epilogue warp
-constexpr size_t kGemmSmem = kTileA + kStages * kChunkB + 512;
-template <Product kMode>
+constexpr size_t kGemmSmem = kTileA + kStages * Geo<8>::kChunkB + 512;
+template <Product kMode, int ND = 8>
 __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
     int ctiles, int coff, int k0, int kb, int nrt, int nct, int cbegin, int kt0, int kskip,
     double* __restrict__ C,
     const char* __restrict__ SA, const int* __restrict__ ea, const char* __restrict__ SB,
     const int* __restrict__ eb, const double* __restrict__ D, DevFlags* flags) {
+  constexpr int kChunks = Geo<ND>::kChunks, kChunkA = Geo<ND>::kChunkA, kChunkB = Geo<ND>::kChunkB;
   extern __shared__ __align__(128) char sm[];
   __shared__ __align__(8) unsigned long long bars[1 + 2 * kStages + 5];
   __shared__ unsigned s_tmem;
@@ -870,14 +916,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
           run = mbar_wait(b_full + 8 * st, (g / kStages) & 1, &s_stop);
           if (!run) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const unsigned long long db = mat_desc(sB + st * kChunkB, (kRowsB / 8) * 128, 128);
-          // digit i of P with the digits 0..7-i of T; digit 0 of the first chunk starts the
-          // eight sums
+          const unsigned long long db = mat_desc(sB + st * kChunkB, (Geo<ND>::kRowsB / 8) * 128, 128);
+          // digit i of P with the digits 0..ND-1-i of T; digit 0 of the first chunk starts the
+          // ND sums
 #pragma unroll
-          for (int i = 0; i < kDigits; ++i)
+          for (int i = 0; i < ND; ++i)
             mma_bf16(tmem + buf * 256 + i * kColTile,
                      mat_desc(sA + c * kChunkA + i * kSliceA, (kRowTile / 8) * 128, 128), db,
-                     kColTile * (kDigits - i), c > 0 || i > 0);
+                     kColTile * (ND - i), c > 0 || i > 0);
           mma_commit(b_empty + 8 * st);
         }
         if (run) mma_commit(b_tfull + 8 * buf);
@@ -945,9 +991,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
       if (!__all_sync(0xffffffffu, run)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       static_assert(kEpiCols == 8, "one load of eight columns per group");
-      unsigned r[kGroups][8];
+      unsigned r[ND][8];
 #pragma unroll
-      for (int m = 0; m < kGroups; ++m)
+      for (int m = 0; m < ND; ++m)
         tmem_ld8(tmem + ((unsigned)(quad * 32) << 16) + buf * 256 + m * kColTile + part * kEpiCols,
                  r[m]);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -955,9 +1001,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
       if (lane == 0) mbar_arrive(b_tempty + 8 * buf);
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        float S[kGroups];
+        float S[ND];
 #pragma unroll
-        for (int m = 0; m < kGroups; ++m) S[m] = __uint_as_float(r[m][c]);
+        for (int m = 0; m < ND; ++m) S[m] = __uint_as_float(r[m][c]);
         const double v = add_digits(S, ev[c], sign, cv[c]);
         if (kMode != kFirst || !in_k) cv[c] = v;
       }
@@ -986,26 +1032,208 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-__global__ void csr_to_dense_kernel(int n, int nct, const int* __restrict__ rp,
-                                    const int* __restrict__ ci, const double* __restrict__ v,
-                                    double* __restrict__ A) {
+// ------------------------------------------------------------------ scaling of the matrix
+// Powers of two r_i, c_j, so that the entries 2^(r_i + c_j) a_ij are of one order of magnitude
+// whatever units the rows and columns of A come in: the digits of an operand share an exponent
+// per row or column, so the products are FP64 products only of rows and columns whose large
+// entries meet.  Six rounds of geometric means (of the entries' binary exponents, as integers:
+// the same on every run), then the largest entry of a row to [0.5, 1).
+constexpr int kScaleRounds = 6;
+__device__ __forceinline__ bool entry_exp(double x, int& e) {
+  if (x == 0.0 || !isfinite(x)) return false;
+  frexp(x, &e);
+  return true;
+}
+// largest: r_i from the largest entry, else from the mean; csum[j], ccnt[j] += exponents, count
+__global__ void row_scale_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                                 const double* __restrict__ v, const int* __restrict__ c, bool largest,
+                                 int* __restrict__ r, int* __restrict__ csum, int* __restrict__ ccnt) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    for (int p = rp[i]; p < rp[i + 1]; ++p) A[tile_at(nct, i, ci[p])] = v[p];
+    int sum = 0, cnt = 0, top = -(1 << 30), e;
+    for (int p = rp[i]; p < rp[i + 1]; ++p)
+      if (entry_exp(v[p], e)) {
+        e += c[ci[p]];
+        sum += e;
+        ++cnt;
+        top = max(top, e);
+      }
+    const int ri = cnt == 0 ? 0 : (largest ? -top : -(int)rint((double)sum / cnt));
+    r[i] = ri;
+    if (largest) continue;
+    for (int p = rp[i]; p < rp[i + 1]; ++p)
+      if (entry_exp(v[p], e)) {
+        atomicAdd(csum + ci[p], e + ri);
+        atomicAdd(ccnt + ci[p], 1);
+      }
+  }
+}
+__global__ void col_scale_kernel(int n, int* __restrict__ csum, int* __restrict__ ccnt, int* __restrict__ c) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    c[j] = ccnt[j] == 0 ? 0 : -(int)rint((double)csum[j] / ccnt[j]);
+    csum[j] = ccnt[j] = 0;
   }
 }
 
-// out (n x n, row-major) = A with its columns in the order colperm: 32 x 32 pieces through
-// shared memory, read along the rows of A's tiles and written along those of out
+// v <- the scaled entries, and A (zeroed) their dense copy
+__global__ void csr_to_dense_kernel(int n, int nct, const int* __restrict__ rp,
+                                    const int* __restrict__ ci, const double* __restrict__ v,
+                                    const int* __restrict__ r, const int* __restrict__ c,
+                                    double* __restrict__ vs, double* __restrict__ A) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int p = rp[i]; p < rp[i + 1]; ++p) {
+      const double x = scalbn(v[p], r[i] + c[ci[p]]);
+      vs[p] = x;
+      A[tile_at(nct, i, ci[p])] = x;
+    }
+  }
+}
+
+// ------------------------------------------------------------------ the correction
+// R = I - B X for the scaled matrix B (CSR) and its inverse X, whose column j stands at place
+// cols[j] of A's tiles (place[cols[j]] = j): R row-major, its columns in the order of the
+// places, and rmax[q] = the largest |R| of a column (as bits).  A block takes 32 rows and 32
+// columns at a time: a lane per row, so that neighbouring rows' entries of X share lines, the
+// piece written along its rows.  n^2 entries of X are read once per stored entry of a row of B
+// (from L2 mostly).
+__global__ void __launch_bounds__(256) inverse_residual_kernel(
+    int n, int nct, const int* __restrict__ rp, const int* __restrict__ ci,
+    const double* __restrict__ vs, const double* __restrict__ X, const int* __restrict__ place,
+    double* __restrict__ R, unsigned long long* __restrict__ rmax) {
+  __shared__ double sh[32][33];
+  const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
+  const int i0 = blockIdx.x * 32, i = i0 + lane;
+  const int p0 = i < n ? rp[i] : 0, p1 = i < n ? rp[i + 1] : 0;
+  for (int ct = blockIdx.y; ct * kColTile < n; ct += gridDim.y) {
+    const int q0 = ct * kColTile;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {  // pairs of columns
+      const int c = (w + 8 * t) * 2;
+      double2 a = make_double2(0.0, 0.0);
+      for (int p = p0; p < p1; ++p) {
+        const double b = -__ldg(vs + p);
+        const double2 x = *reinterpret_cast<const double2*>(X + tile_at(nct, __ldg(ci + p), q0 + c));
+        a.x = fma(b, x.x, a.x);
+        a.y = fma(b, x.y, a.y);
+      }
+      const bool h0 = i < n && q0 + c < n, h1 = i < n && q0 + c + 1 < n;
+      if (h0 && place[q0 + c] == i) a.x += 1.0;
+      if (h1 && place[q0 + c + 1] == i) a.y += 1.0;
+      sh[lane][c] = h0 ? a.x : 0.0;
+      sh[lane][c + 1] = h1 ? a.y : 0.0;
+    }
+    __syncthreads();
+    if (w == 0 && q0 + lane < n) {
+      unsigned long long m = 0;
+      for (int r = 0; r < 32; ++r) {
+        const unsigned long long b =
+            (unsigned long long)__double_as_longlong(sh[r][lane]) & 0x7fffffffffffffffULL;
+        m = b > m ? b : m;  // a NaN is larger than any number
+      }
+      atomicMax(rmax + q0 + lane, m);
+    }
+    for (int r = w; r < 32; r += 8)
+      if (i0 + r < n && q0 + lane < n) R[(size_t)(i0 + r) * n + q0 + lane] = sh[r][lane];
+    __syncthreads();
+  }
+}
+
+// Six digits of the columns k0..k0+127 of X (at the places cols[k0..]) for 16 rows a block
+constexpr int kCorrK = CorrGeo::kK;
+constexpr int kCorrRows = 16;
+__global__ void __launch_bounds__(256) slice_inverse_kernel(int n, int nct, int k0,
+                                                            const double* __restrict__ X,
+                                                            const int* __restrict__ cols,
+                                                            char* __restrict__ S, int* __restrict__ exps) {
+  __shared__ double sh[kCorrRows][kCorrK + 1];
+  __shared__ int se[kCorrRows];
+  const int r0 = blockIdx.x * kCorrRows;
+  for (int t = threadIdx.x; t < kCorrRows * kCorrK; t += 256) {
+    const int r = t % kCorrRows, q = t / kCorrRows;
+    sh[r][q] = k0 + q < n ? X[tile_at(nct, r0 + r, __ldg(cols + k0 + q))] : 0.0;
+  }
+  __syncthreads();
+  {
+    const int r = threadIdx.x / 16, l = threadIdx.x % 16;  // sixteen lanes per row
+    double m = 0.0;
+    bool bad = false;
+    for (int q = l; q < kCorrK; q += 16) {
+      const double a = fabs(sh[r][q]);
+      bad |= !isfinite(a);
+      m = fmax(m, a);
+    }
+    if (bad) m = __longlong_as_double(0x7ff0000000000000LL);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o, 16));
+    if (l == 0) {
+      const int e = scale_exp(m);
+      se[r] = e;
+      exps[r0 + r] = e;
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < kCorrRows * (kCorrK / 8); t += 256) {
+    const int r = t % kCorrRows, kcg = t / kCorrRows;
+    double x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = sh[r][kcg * 8 + q];
+    store_digits8<kCorrDigits>(x, se[r], digit_a<kCorrDigits>(S, r0 + r, kcg), kSliceA);
+  }
+}
+
+// Six digits of the rows k0..k0+127 of R, a tile of 32 columns a block.  A column whose
+// residual is not small (an inverse without correct digits, or not finite) is left as it is.
+constexpr double kCorrLimit = 0.0078125;
+__global__ void __launch_bounds__(256) slice_residual_kernel(int n, int k0, const double* __restrict__ R,
+                                                             const unsigned long long* __restrict__ rmax,
+                                                             char* __restrict__ S, int* __restrict__ exps) {
+  extern __shared__ double swap_smem[];  // [kCorrK][33]
+  double(*sh)[kColTile + 1] = reinterpret_cast<double(*)[kColTile + 1]>(swap_smem);
+  __shared__ double smax[8][kColTile];
+  __shared__ int se[kColTile];
+  const int ct = blockIdx.x, lane = threadIdx.x % 32, w = threadIdx.x / 32;
+  const int c = ct * kColTile + lane;
+  const bool use = c < n && __longlong_as_double((long long)rmax[c < n ? c : 0]) <= kCorrLimit;
+  double m = 0.0;
+  for (int q = w; q < kCorrK; q += 8) {
+    const double x = use && k0 + q < n ? R[(size_t)(k0 + q) * n + c] : 0.0;
+    sh[q][lane] = x;
+    m = fmax(m, fabs(x));
+  }
+  smax[w][lane] = m;
+  __syncthreads();
+  if (w == 0) {
+    for (int u = 1; u < 8; ++u) m = fmax(m, smax[u][lane]);
+    const int e = scale_exp(m);
+    se[lane] = e;
+    exps[c] = e;
+  }
+  __syncthreads();
+  char* tile = S + (size_t)ct * kTileB;
+  for (int t = threadIdx.x; t < kColTile * (kCorrK / 8); t += 256) {
+    const int cc = t % kColTile, kcg = t / kColTile;
+    double x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = sh[kcg * 8 + q][cc];
+    store_digits8<kCorrDigits>(x, se[cc], digit_b<kCorrDigits>(tile, cc, kcg), CorrGeo::kDigitB);
+  }
+}
+
+// out (n x n, row-major) = A with its columns in the order colperm, the scaling undone: 32 x 32
+// pieces through shared memory, read along the rows of A's tiles and written along those of out
 __global__ void __launch_bounds__(256) unscramble_kernel(int n, int nct,
                                                          const int* __restrict__ colperm,
                                                          const double* __restrict__ A,
+                                                         const int* __restrict__ rs,
+                                                         const int* __restrict__ cs,
                                                          double* __restrict__ out) {
   __shared__ double sh[32][33];
   const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
   const int i0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
 #pragma unroll
   for (int c = w; c < 32; c += 8)
-    sh[lane][c] = (i0 + lane < n && c0 + c < n) ? A[tile_at(nct, i0 + lane, colperm[c0 + c])] : 0.0;
+    sh[lane][c] = (i0 + lane < n && c0 + c < n)
+                      ? scalbn(A[tile_at(nct, i0 + lane, colperm[c0 + c])], cs[i0 + lane] + rs[c0 + c])
+                      : 0.0;
   __syncthreads();
 #pragma unroll
   for (int r = w; r < 32; r += 8)
@@ -1073,7 +1301,7 @@ struct SideStream {
 
 }  // namespace
 
-int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v, double* out,
+int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const double* v, double* out,
                            DevFlags* flags, cudaStream_t s) {
   if (n <= 0) return MSP_ERR_ARG;
   const int lda = (int)(div_up(n, kP) * kP), nrt = (int)div_up(n, kRowTile);
@@ -1081,7 +1309,9 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
   const size_t rows = (size_t)nrt * kRowTile;
   DevBuf<double> A, X, Y, D;
   DevBuf<char> SA, ST, SD;
-  DevBuf<int> ea, et, ed, piv, pivots, perm, cols_d;
+  DevBuf<double> vs;
+  DevBuf<int> ea, et, ed, piv, pivots, perm, cols_d, rs, cs, csum;
+  DevBuf<unsigned long long> rmax;
   MSP_TRY(A.alloc(rows * lda));
   MSP_TRY(X.alloc((size_t)n * kP));
   MSP_TRY(Y.alloc(rows * kP));
@@ -1095,15 +1325,31 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
   MSP_TRY(piv.alloc(kP));
   MSP_TRY(pivots.alloc((size_t)lda));
   MSP_TRY(perm.alloc(1 + 4 * kP));
-  MSP_TRY(cols_d.alloc(n));
+  MSP_TRY(cols_d.alloc(2 * (size_t)n));
+  MSP_TRY(vs.alloc((size_t)nnz));
+  MSP_TRY(rs.alloc(n));
+  MSP_TRY(cs.alloc(n));
+  MSP_TRY(csum.alloc(2 * (size_t)n));
+  MSP_TRY(rmax.alloc(n));
+  MSP_CUDA_TRY(cudaMemsetAsync(cs.p, 0, n * sizeof(int), s));
+  MSP_CUDA_TRY(cudaMemsetAsync(csum.p, 0, 2 * (size_t)n * sizeof(int), s));
+  MSP_CUDA_TRY(cudaMemsetAsync(rmax.p, 0, n * sizeof(unsigned long long), s));
   MSP_CUDA_TRY(cudaMemsetAsync(A.p, 0, rows * lda * sizeof(double), s));
-  csr_to_dense_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, act, rp, ci, v, A.p);
+  for (int round = 0; round <= kScaleRounds; ++round) {
+    row_scale_kernel<<<grid_for(n, 128), 128, 0, s>>>(n, rp, ci, v, cs.p, round == kScaleRounds, rs.p,
+                                                      csum.p, csum.p + n);
+    MSP_TRY(launch_status());
+    if (round == kScaleRounds) break;
+    col_scale_kernel<<<grid_for(n, 128), 128, 0, s>>>(n, csum.p, csum.p + n, cs.p);
+    MSP_TRY(launch_status());
+  }
+  csr_to_dense_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, act, rp, ci, v, rs.p, cs.p, vs.p, A.p);
   MSP_TRY(launch_status());
   const size_t diag_smem = sizeof(double) * (kP * (kP + 1) + kP);
   MSP_CUDA_TRY(cudaFuncSetAttribute(diag_inverse_panel_kernel,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem));
   for (auto* k : {slice_gemm_kernel<kUpdate>, slice_gemm_kernel<kFirst>, slice_gemm_kernel<kResid>,
-                  slice_gemm_kernel<kCorrect>})
+                  slice_gemm_kernel<kCorrect>, slice_gemm_kernel<kResid, kCorrDigits>})
     MSP_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)kGemmSmem));
   const size_t swap_smem = sizeof(double) * 2 * kP * (kColTile + 1);
@@ -1189,7 +1435,7 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
     MSP_TRY(update(nct - nown - nnext, 0, kt0, nown + nnext,
                    nnext > 0 ? std::max(1, sm_count() - kMaxCluster) : sm_count()));
   }
-  std::vector<int> hp(n), cols(n);
+  std::vector<int> hp(n), cols(n), place(n);
   DevFlags hf{};
   MSP_CUDA_TRY(cudaMemcpyAsync(hp.data(), pivots.p, n * sizeof(int), cudaMemcpyDeviceToHost, s));
   MSP_CUDA_TRY(cudaMemcpyAsync(&hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, s));
@@ -1198,11 +1444,35 @@ int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v,
   for (int c = 0; c < n; ++c) cols[c] = c;
   for (int k = n - 1; k >= 0; --k)
     if (hp[k] != k) std::swap(cols[k], cols[hp[k]]);
+  for (int c = 0; c < n; ++c) place[cols[c]] = c;
+  const int* cols_p = cols_d.p;
+  const int* place_p = cols_d.p + n;
   MSP_CUDA_TRY(cudaMemcpyAsync(cols_d.p, cols.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
-  unscramble_kernel<<<dim3(div_up(n, 32), div_up(n, 32)), 256, 0, s>>>(n, act, cols_d.p, A.p, out);
+  MSP_CUDA_TRY(cudaMemcpyAsync(cols_d.p + n, place.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
+  // X += X (I - B X), the residual in `out` until the end; 128 columns of X a step, which see
+  // the steps before theirs (a second-order change)
+  inverse_residual_kernel<<<dim3(div_up(n, 32), std::min(nct, 16)), 256, 0, s>>>(
+      n, act, rp, ci, vs.p, A.p, place_p, out, rmax.p);
   MSP_TRY(launch_status());
+  const size_t corr_smem = sizeof(double) * kCorrK * (kColTile + 1);
+  MSP_CUDA_TRY(cudaFuncSetAttribute(slice_residual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)corr_smem));
+  for (int k0 = 0; k0 < n; k0 += kCorrK) {
+    slice_inverse_kernel<<<(unsigned)(rows / kCorrRows), 256, 0, s>>>(n, act, k0, A.p, cols_p, SA.p, ea.p);
+    MSP_TRY(launch_status());
+    slice_residual_kernel<<<nct, 256, corr_smem, s>>>(n, k0, out, rmax.p, ST.p, et.p);
+    MSP_TRY(launch_status());
+    slice_gemm_kernel<kResid, kCorrDigits><<<(unsigned)std::min<long long>(sm_count(), (long long)nrt * nct),
+                                   kGemmThreads, kGemmSmem, s>>>(
+        act, 0, 0, 0, nrt, nct, 0, 0, 0, A.p, SA.p, ea.p, ST.p, et.p, D.p, flags);
+    MSP_TRY(launch_status());
+  }
+  unscramble_kernel<<<dim3(div_up(n, 32), div_up(n, 32)), 256, 0, s>>>(n, act, cols_p, A.p, rs.p, cs.p,
+                                                                       out);
+  MSP_TRY(launch_status());
+  MSP_CUDA_TRY(cudaMemcpyAsync(&hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, s));
   MSP_CUDA_TRY(cudaStreamSynchronize(s));  // cols and the temporaries are in use until here
-  return MSP_OK;
+  return hf.code;
 }
 
 }  // namespace msp

@@ -768,7 +768,7 @@ int level_extras(msp_handle h, Level& L, bool smoothed, bool ell, cudaStream_t s
 int coarse_inverse(msp_handle h, const DCsr& C, cudaStream_t s) {
   const int n = C.n;
   MSP_TRY(h->cinv.alloc((size_t)n * n));
-  MSP_TRY(coarse_inverse_blocked(n, C.rp.p, C.ci.p, C.v.p, h->cinv.p, h->flags.p, s));
+  MSP_TRY(coarse_inverse_blocked(n, C.nnz, C.rp.p, C.ci.p, C.v.p, h->cinv.p, h->flags.p, s));
   h->ncoarse = n;
   return MSP_OK;
 }

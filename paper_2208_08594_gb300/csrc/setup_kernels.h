@@ -107,7 +107,7 @@ int launch_bilu_factor(int b, int r0, int r1, const int* rp, const int* ci, cons
                        double* lu, double* uinv, DevFlags* flags, cudaStream_t s);
 // out (n x n, row-major) = the inverse of a CSR matrix, in FP64 (coarse_inverse.cu);
 // MSP_ERR_SINGULAR_BLOCK where a column has no nonzero pivot.  Synchronises the stream.
-int coarse_inverse_blocked(int n, const int* rp, const int* ci, const double* v, double* out,
+int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const double* v, double* out,
                            DevFlags* flags, cudaStream_t s);
 int launch_cast_vals(size_t n, const double* in, float* out, cudaStream_t s);
 int launch_iota(int n, int* out, cudaStream_t s);

@@ -103,3 +103,65 @@ def test_singular_coarsest_matrix_is_reported():
         msp.Solver(n, 1, torch.from_numpy(rp).to(DEV), torch.from_numpy(cols.astype(np.int32)).to(DEV),
                    torch.from_numpy(a[rows, cols]).to(DEV), coarse_max=20000, colouring=msp.MSP_COLOURING_JP)
     assert e.value.status == msp._native.MSP_ERR_SINGULAR_BLOCK
+
+
+def _grid(nx, ny, nz, sigma, seed):
+    """7-point matrix with lognormal permeability exp(sigma N), rows with unit diagonals."""
+    rng = np.random.default_rng(seed)
+    n = nx * ny * nz
+    k = np.exp(sigma * rng.normal(size=(nz, ny, nx)))
+    idx, a = np.arange(n).reshape(nz, ny, nx), np.zeros((n, n))
+    for ax in range(3):
+        i, kk = np.moveaxis(idx, ax, 0), np.moveaxis(k, ax, 0)
+        t = (2 * kk[1:] * kk[:-1] / (kk[1:] + kk[:-1])).ravel()
+        a[i[1:].ravel(), i[:-1].ravel()] = -t * rng.uniform(0.1, 1, t.size)
+        a[i[:-1].ravel(), i[1:].ravel()] = -t * rng.uniform(0.1, 1, t.size)
+    a[np.arange(n), np.arange(n)] = rng.uniform(0.5, 2.0, n) - a.sum(1)
+    return a / np.diag(a)[:, None]
+
+
+SCALES = {  # binary exponents of the rows and of the columns
+    "unit": lambda rng, n: (np.zeros(n, int), np.zeros(n, int)),
+    "last_rows_up": lambda rng, n: (np.where(np.arange(n) >= n - 4, 33, 0), np.zeros(n, int)),
+    "last_rows_down": lambda rng, n: (np.where(np.arange(n) >= n - 4, -33, 0), np.zeros(n, int)),
+    "first_rows_up": lambda rng, n: (np.where(np.arange(n) < 3, 47, 0), np.zeros(n, int)),
+    "last_unknowns": lambda rng, n: (np.zeros(n, int), np.where(np.arange(n) >= n - 4, -33, 0)),
+    "rows": lambda rng, n: (rng.integers(-30, 31, n), np.zeros(n, int)),
+    "columns": lambda rng, n: (np.zeros(n, int), rng.integers(-30, 31, n)),
+    "both": lambda rng, n: (rng.integers(-30, 31, n), rng.integers(-30, 31, n)),
+    "tiny": lambda rng, n: (np.full(n, -900), np.zeros(n, int)),
+    "huge": lambda rng, n: (np.full(n, 900), np.zeros(n, int)),
+}
+
+
+@pytest.mark.parametrize("scale", sorted(SCALES))
+@pytest.mark.parametrize("matrix", ["grid", "spread_grid", "exchanges"])
+def test_rows_and_columns_in_other_units(matrix, scale):
+    """Without the decoupling weights the coarsest rows keep the units of the caller's rows.
+    A = 2^r A0 2^c has the inverse 2^-c A0^-1 2^-r exactly, and elimination in FP64 keeps
+    |E| <= n 2^-53 |A^-1| |A| |A^-1| entry by entry (times a small factor) for all of them, as
+    does one step of refinement in the working precision: the same bound, with a factor of 8
+    for the inverse and 8 for the reference (an FP64 inverse of A0 and such a step), for whole
+    vectors and for single columns of the inverse, whose entries span ten orders of magnitude."""
+    if matrix == "exchanges":
+        a0 = _dense(*_system(300, 7, True), 300)
+    else:
+        a0 = _grid(8, 7, 6, 4.0 if matrix == "spread_grid" else 1.0, 3)
+    n = len(a0)
+    rng = np.random.default_rng(11)
+    r, c = SCALES[scale](rng, n)
+    a = np.ldexp(np.ldexp(a0, r[:, None]), c[None, :])
+    x0 = np.linalg.inv(a0)
+    x0 += x0 @ (np.eye(n) - a0 @ x0)
+    bound = 16.0 * n * 2.0 ** -53 * (np.abs(x0) @ np.abs(a0) @ np.abs(x0))
+    rows, cols = np.nonzero(a)
+    rp = np.searchsorted(rows, np.arange(n + 1)).astype(np.int32)
+    s = msp.Solver(n, 1, *(torch.from_numpy(x).to(DEV) for x in (rp, cols.astype(np.int32), a[rows, cols])),
+                   coarse_max=20000, precond=msp.MSP_PREC_P_ONLY, colouring=msp.MSP_COLOURING_JP, decoupling=0)
+    assert s.num_levels == 1
+    for g in [rng.normal(size=n)] + [np.eye(n)[j] for j in (0, n // 2, n - 5, n - 1)]:
+        w = torch.empty(n, dtype=torch.float64, device=DEV)
+        s.apply_precond(torch.from_numpy(np.ldexp(g, r)).to(DEV), w)
+        x = np.ldexp(w.cpu().numpy(), c)
+        assert (np.abs(x - x0 @ g) <= bound @ np.abs(g)).all()
+    s.close()
