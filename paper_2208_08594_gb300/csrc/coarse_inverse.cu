@@ -1242,14 +1242,15 @@ __global__ void __launch_bounds__(256) unscramble_kernel(int n, int nct,
 
 // The sub-panels of one step: LU of the m x kb panel copy X.
 template <int W, int R>
-int lu_panel(int m, int kb, int k0, double* X, int* piv, DevFlags* flags, cudaStream_t s) {
+int lu_panel(int m, int kb, int k0, int cluster, double* X, int* piv, DevFlags* flags,
+             cudaStream_t s) {
   MSP_CUDA_TRY(cudaFuncSetAttribute(lu_panel_kernel<W, R>,
                                     cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   for (int c0 = 0; c0 < kb; c0 += W) {
     const int w = std::min(W, kb - c0), rows = m - c0;
     // about 128 rows per CTA: more CTAs make the barrier dearer, fewer the rank-1 updates
     int nct = 1;
-    while (nct < kMaxCluster && nct * 128 < rows) nct *= 2;
+    while (nct < cluster && nct * 128 < rows) nct *= 2;
     const int rpc = std::max(W, (rows + nct - 1) / nct);  // CTA 0 holds the rows c0..c0+w-1
     const int threads = std::max(kP, (int)div_up(div_up(rpc, R), kWarp) * kWarp);
     if (threads > kLuThreads) return MSP_ERR_ARG;
@@ -1271,6 +1272,29 @@ int lu_panel(int m, int kb, int k0, double* X, int* piv, DevFlags* flags, cudaSt
       MSP_TRY(launch_status());
     }
   }
+  return MSP_OK;
+}
+
+// CTAs of the panels' cluster: 16 is past the portable size, so the device is asked whether it
+// can place one (of 512 threads and all their registers: a whole SM each); 8 always fit
+int panel_cluster(int* out) {
+  MSP_CUDA_TRY(cudaFuncSetAttribute(lu_panel_kernel<16, 1>,
+                                    cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kMaxCluster);
+  cfg.blockDim = dim3(kLuThreads);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kMaxCluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int fit = 0;
+  if (cudaOccupancyMaxActiveClusters(&fit, lu_panel_kernel<16, 1>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    fit = 0;
+  }
+  *out = fit > 0 ? kMaxCluster : 8;
   return MSP_OK;
 }
 
@@ -1302,8 +1326,11 @@ struct SideStream {
 }  // namespace
 
 int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const double* v, double* out,
-                           DevFlags* flags, cudaStream_t s) {
+                           DevFlags* flags, cudaStream_t s, const InverseOptions& opt) {
   if (n <= 0) return MSP_ERR_ARG;
+  int cluster = opt.cluster;
+  if (cluster == 0) MSP_TRY(panel_cluster(&cluster));
+  if (cluster < 1 || cluster > kMaxCluster) return MSP_ERR_ARG;
   const int lda = (int)(div_up(n, kP) * kP), nrt = (int)div_up(n, kRowTile);
   const int nct = (int)div_up(n, kColTile), act = lda / kColTile;  // column tiles used, stored
   const size_t rows = (size_t)nrt * kRowTile;
@@ -1371,15 +1398,18 @@ int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const d
     MSP_TRY(launch_status());
     MSP_CUDA_TRY(cudaEventRecord(side.copied, f));
     // the widest sub-panel whose rows fit the registers of one cluster
-    constexpr int kLuRows = kMaxCluster * kLuThreads;
-    if (m <= kLuRows)
-      MSP_TRY((lu_panel<16, 1>(m, kb, k0, X.p, piv.p, flags, f)));
-    else if (m <= 2 * kLuRows)
-      MSP_TRY((lu_panel<8, 2>(m, kb, k0, X.p, piv.p, flags, f)));
-    else if (m <= 4 * kLuRows)
-      MSP_TRY((lu_panel<4, 4>(m, kb, k0, X.p, piv.p, flags, f)));
-    else if (m <= 16 * kLuRows)
-      MSP_TRY((lu_panel<2, 16>(m, kb, k0, X.p, piv.p, flags, f)));
+    const int fits = (int)div_up(m, (size_t)cluster * kLuThreads);  // rows a thread
+    const int r = std::max(fits, opt.panel_rows);
+    if (r <= 1)
+      MSP_TRY((lu_panel<16, 1>(m, kb, k0, cluster, X.p, piv.p, flags, f)));
+    else if (r <= 2)
+      MSP_TRY((lu_panel<8, 2>(m, kb, k0, cluster, X.p, piv.p, flags, f)));
+    else if (r <= 4)
+      MSP_TRY((lu_panel<4, 4>(m, kb, k0, cluster, X.p, piv.p, flags, f)));
+    else if (r <= 16)
+      MSP_TRY((lu_panel<2, 16>(m, kb, k0, cluster, X.p, piv.p, flags, f)));
+    else if (r <= 32)
+      MSP_TRY((lu_panel<2, 32>(m, kb, k0, cluster, X.p, piv.p, flags, f)));
     else
       return MSP_ERR_NOMEM;  // two dense copies of such a matrix exceed the device
     diag_inverse_panel_kernel<<<kP / kDiagWarps + 1, kDiagWarps * kWarp, diag_smem, f>>>(
@@ -1433,7 +1463,7 @@ int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const d
       MSP_CUDA_TRY(cudaStreamWaitEvent(s, side.copied, 0));
     }
     MSP_TRY(update(nct - nown - nnext, 0, kt0, nown + nnext,
-                   nnext > 0 ? std::max(1, sm_count() - kMaxCluster) : sm_count()));
+                   nnext > 0 ? std::max(1, sm_count() - cluster) : sm_count()));
   }
   std::vector<int> hp(n), cols(n), place(n);
   DevFlags hf{};
@@ -1476,3 +1506,19 @@ int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const d
 }
 
 }  // namespace msp
+
+// For tests of the variants that a whole GPU or a small matrix never takes: the inverse of a
+// CSR matrix (device arrays) with panels of `cluster` CTAs and at least panel_rows rows a thread.
+// Not part of the interface.
+extern "C" int msp_test_inverse(int32_t n, int32_t nnz, const int32_t* d_rp, const int32_t* d_ci,
+                                const double* d_v, double* d_out, int32_t cluster, int32_t panel_rows,
+                                void* stream) {
+  using namespace msp;
+  DevBuf<DevFlags> flags;
+  MSP_TRY(flags.alloc(1));
+  MSP_CUDA_TRY(cudaMemsetAsync(flags.p, 0, sizeof(DevFlags), (cudaStream_t)stream));
+  InverseOptions opt;
+  opt.cluster = cluster;
+  opt.panel_rows = panel_rows;
+  return coarse_inverse_blocked(n, nnz, d_rp, d_ci, d_v, d_out, flags.p, (cudaStream_t)stream, opt);
+}

@@ -105,10 +105,15 @@ int launch_rdiag(int n, const int* dpos, const double* v, double* rdiag, DevFlag
 // BILU(0) factorisation of the rows [r0, r1) of one colour (rows of earlier colours done)
 int launch_bilu_factor(int b, int r0, int r1, const int* rp, const int* ci, const int* dpos,
                        double* lu, double* uinv, DevFlags* flags, cudaStream_t s);
+struct InverseOptions {
+  int cluster = 0;     // CTAs of the panels' cluster (0: as many as the device places, 16 or 8)
+  int panel_rows = 0;  // at least this many rows of the panel a thread (for tests)
+};
 // out (n x n, row-major) = the inverse of a CSR matrix, in FP64 (coarse_inverse.cu);
 // MSP_ERR_SINGULAR_BLOCK where a column has no nonzero pivot.  Synchronises the stream.
 int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const double* v, double* out,
-                           DevFlags* flags, cudaStream_t s);
+                           DevFlags* flags, cudaStream_t s,
+                           const InverseOptions& opt = InverseOptions());
 int launch_cast_vals(size_t n, const double* in, float* out, cudaStream_t s);
 int launch_iota(int n, int* out, cudaStream_t s);
 int launch_fill_int(size_t n, int value, int* out, cudaStream_t s);
