@@ -712,11 +712,28 @@ __device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes) {
 __device__ __forceinline__ void mbar_arrive(unsigned bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// Wait for the phase of the given parity, with a limit; false (and the block's stop word
-// set) when the limit runs out or another warp has stopped.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* stop) {
-  for (int it = 0; it < (1 << 20); ++it) {
-    unsigned done;
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+// Wait for the phase of the given parity for at most limit_ns (and 2^20 attempts); false (and
+// the block's stop word set) when the limit runs out or another warp has stopped.  The first
+// look does not suspend the thread, so that a limit of 0 gives up wherever there is a wait.
+constexpr unsigned long long kWaitNs = InverseOptions::kWaitNs;
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* stop,
+                                          unsigned long long limit_ns) {
+  unsigned done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  if (done) return true;
+  const unsigned long long t0 = now_ns();
+  for (int it = 0; it < (1 << 20) && limit_ns > 0; ++it) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -726,6 +743,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatil
         : "memory");
     if (done) return true;
     if (*stop) return false;
+    if (now_ns() - t0 > limit_ns) break;
   }
   *stop = 1;
   return false;
@@ -828,7 +846,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
     int ctiles, int coff, int k0, int kb, int nrt, int nct, int cbegin, int kt0, int kskip,
     double* __restrict__ C,
     const char* __restrict__ SA, const int* __restrict__ ea, const char* __restrict__ SB,
-    const int* __restrict__ eb, const double* __restrict__ D, DevFlags* flags) {
+    const int* __restrict__ eb, const double* __restrict__ D, DevFlags* flags,
+    unsigned long long wait_ns) {
   constexpr int kChunks = Geo<ND>::kChunks, kChunkA = Geo<ND>::kChunkA, kChunkB = Geo<ND>::kChunkB;
   extern __shared__ __align__(128) char sm[];
   __shared__ __align__(8) unsigned long long bars[1 + 2 * kStages + 5];
@@ -840,7 +859,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
   const unsigned b_a = smem_u32(&bars[0]);
   const unsigned b_full = smem_u32(&bars[1]), b_empty = smem_u32(&bars[1 + kStages]);
   const unsigned b_tfull = smem_u32(&bars[1 + 2 * kStages]), b_tempty = b_tfull + 16;
-  const unsigned b_end = b_tempty + 16;  // used only after a stop
+  const unsigned b_end = b_tempty + 16;  // every MMA issued
   const long long total = (long long)nrt * nct;
   const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
   if (threadIdx.x == 0) {
@@ -872,6 +891,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
     if (lane == 0) {
       int prev = -1;
       unsigned g = 0;  // chunks so far: buffer g % kStages, its use g / kStages
+      unsigned na = 0;  // row tiles so far
       bool run = true;
       for (long long t = t0; t < t1 && run; ++t) {
         const int rt = (int)(t / nct), q = (int)(t % nct);
@@ -879,8 +899,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
         if (rt != prev) {
           // the previous row tile's digits are free once its last chunk has been used
           if (g > 0)
-            run = mbar_wait(b_empty + 8 * ((g - 1) % kStages), ((g - 1) / kStages) & 1, &s_stop);
+            run = mbar_wait(b_empty + 8 * ((g - 1) % kStages), ((g - 1) / kStages) & 1, &s_stop, wait_ns);
           if (!run) break;
+          ++na;
           mbar_expect(b_a, kTileA);
           for (int c = 0; c < kChunks; ++c)
             bulk_load(sA + c * kChunkA, SA + (size_t)rt * kTileA + (size_t)c * kChunkA, kChunkA, b_a);
@@ -888,13 +909,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
         }
         for (int c = 0; c < kChunks && run; ++c, ++g) {
           const unsigned st = g % kStages;
-          if (g >= kStages) run = mbar_wait(b_empty + 8 * st, ((g / kStages) - 1) & 1, &s_stop);
+          if (g >= kStages) run = mbar_wait(b_empty + 8 * st, ((g / kStages) - 1) & 1, &s_stop, wait_ns);
           if (!run) break;
           mbar_expect(b_full + 8 * st, kChunkB);
           bulk_load(sB + st * kChunkB, SB + (size_t)ct * kTileB + (size_t)c * kChunkB, kChunkB,
                     b_full + 8 * st);
         }
       }
+      // the copies in flight land before the block (and its shared memory) goes away, whoever
+      // stopped: the last phase of each barrier that has a copy
+      volatile int never = 0;
+      if (na > 0) mbar_wait(b_a, (na - 1) & 1, &never, kWaitNs);
+      for (unsigned q = g > kStages ? g - kStages : 0; q < g; ++q)
+        mbar_wait(b_full + 8 * (q % kStages), (q / kStages) & 1, &never, kWaitNs);
     }
   } else if (wid == kEpiWarps + 1) {
     if (lane == 0) {
@@ -904,16 +931,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
       for (long long t = t0; t < t1 && run; ++t, ++it) {
         const int rt = (int)(t / nct);
         if (rt != prev) {
-          run = mbar_wait(b_a, na & 1, &s_stop);
+          run = mbar_wait(b_a, na & 1, &s_stop, wait_ns);
           ++na;
           prev = rt;
         }
         const unsigned buf = it & 1;
-        if (run && it >= 2) run = mbar_wait(b_tempty + 8 * buf, ((it >> 1) - 1) & 1, &s_stop);
+        if (run && it >= 2) run = mbar_wait(b_tempty + 8 * buf, ((it >> 1) - 1) & 1, &s_stop, wait_ns);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         for (int c = 0; c < kChunks && run; ++c, ++g) {
           const unsigned st = g % kStages;
-          run = mbar_wait(b_full + 8 * st, (g / kStages) & 1, &s_stop);
+          run = mbar_wait(b_full + 8 * st, (g / kStages) & 1, &s_stop, wait_ns);
           if (!run) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const unsigned long long db = mat_desc(sB + st * kChunkB, (Geo<ND>::kRowsB / 8) * 128, 128);
@@ -928,13 +955,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
         }
         if (run) mma_commit(b_tfull + 8 * buf);
       }
-      // every MMA issued here ends before the accumulators and the buffers go away: the
-      // epilogue warps wait for all of them, and after a stop this waits for a commit
-      if (!run) {
-        volatile int never = 0;
-        mma_commit(b_end);
-        mbar_wait(b_end, 0, &never);
-      }
+      // every MMA issued here ends before the accumulators and the buffers go away, also where
+      // an epilogue warp has stopped
+      volatile int never = 0;
+      mma_commit(b_end);
+      mbar_wait(b_end, 0, &never, kWaitNs);
     }
   } else {
     const int quad = wid & 3, part = wid >> 2;  // a warp reads the TMEM lanes of its quadrant
@@ -987,7 +1012,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
       }
       if (t + 1 < t1) load_c(t + 1, cn);
       const unsigned buf = it & 1;
-      const bool run = mbar_wait(b_tfull + 8 * buf, (it >> 1) & 1, &s_stop);
+      const bool run = mbar_wait(b_tfull + 8 * buf, (it >> 1) & 1, &s_stop, wait_ns);
       if (!__all_sync(0xffffffffu, run)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       static_assert(kEpiCols == 8, "one load of eight columns per group");
@@ -1013,19 +1038,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) slice_gemm_kernel(
     }
   }
   __syncthreads();
-  if (s_stop) {
-    // a wait ran out: the copies in flight land before the block (and its shared memory)
-    // goes away; the last expected phase of every chunk is waited for, with a limit
-    if (threadIdx.x == 0) {
-      raise_flag(flags, MSP_ERR_TIMEOUT, blockIdx.x);
-      volatile int never = 0;
-      for (int par = 0; par < 2; ++par) {
-        mbar_wait(b_a, par, &never);
-        for (int c = 0; c < kStages; ++c) mbar_wait(b_full + 8 * c, par, &never);
-      }
-    }
-    __syncthreads();
-  }
+  if (s_stop && threadIdx.x == 0) raise_flag(flags, MSP_ERR_TIMEOUT, blockIdx.x);  // a wait ran out
   __syncwarp();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (wid == kEpiWarps + 1)
@@ -1430,17 +1443,17 @@ int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const d
     slice_rows_kernel<<<srow, 256, 0, s>>>(act, k0, k0, k0 + kb, A.p, SA.p, ea.p, Y.p);
     MSP_TRY(launch_status());
     slice_gemm_kernel<kFirst><<<pt, kGemmThreads, kGemmSmem, s>>>(
-        act, kt0, k0, kb, nrt, kKTiles, 0, 0, 0, A.p, SA.p, ea.p, SD.p, ed.p, D.p, flags);
+        act, kt0, k0, kb, nrt, kKTiles, 0, 0, 0, A.p, SA.p, ea.p, SD.p, ed.p, D.p, flags, opt.wait_ns);
     MSP_TRY(launch_status());
     slice_rows_kernel<<<srow, 256, 0, s>>>(act, k0, 0, 0, A.p, SA.p, ea.p, nullptr);
     MSP_TRY(launch_status());
     slice_gemm_kernel<kResid><<<pt, kGemmThreads, kGemmSmem, s>>>(
-        kKTiles, 0, k0, kb, nrt, kKTiles, 0, 0, 0, Y.p, SA.p, ea.p, SK, et.p + k0, D.p, flags);
+        kKTiles, 0, k0, kb, nrt, kKTiles, 0, 0, 0, Y.p, SA.p, ea.p, SK, et.p + k0, D.p, flags, opt.wait_ns);
     MSP_TRY(launch_status());
     slice_rows_kernel<<<srow, 256, 0, s>>>(kKTiles, 0, 0, 0, Y.p, SA.p, ea.p, nullptr);
     MSP_TRY(launch_status());
     slice_gemm_kernel<kCorrect><<<pt, kGemmThreads, kGemmSmem, s>>>(
-        act, kt0, k0, kb, nrt, kKTiles, 0, 0, 0, A.p, SA.p, ea.p, SD.p, ed.p, D.p, flags);
+        act, kt0, k0, kb, nrt, kKTiles, 0, 0, 0, A.p, SA.p, ea.p, SD.p, ed.p, D.p, flags, opt.wait_ns);
     MSP_TRY(launch_status());
     const int nown = std::min(nct - kt0, kKTiles), nnext = std::min(nct - kt0 - nown, kKTiles);
     if (nct - nown <= 0) continue;
@@ -1451,7 +1464,7 @@ int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const d
       if (tiles <= 0) return MSP_OK;
       slice_gemm_kernel<kUpdate><<<(unsigned)std::min<long long>(blocks, tiles), kGemmThreads,
                                    kGemmSmem, s>>>(act, 0, k0, kb, nrt, count, cbegin, skip_at, skip,
-                                                   A.p, SA.p, ea.p, ST.p, et.p, D.p, flags);
+                                                   A.p, SA.p, ea.p, ST.p, et.p, D.p, flags, opt.wait_ns);
       return launch_status();
     };
     MSP_TRY(update(nnext, kt0 + nown, nnext, 0, sm_count()));
@@ -1494,7 +1507,7 @@ int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const d
     MSP_TRY(launch_status());
     slice_gemm_kernel<kResid, kCorrDigits><<<(unsigned)std::min<long long>(sm_count(), (long long)nrt * nct),
                                    kGemmThreads, kGemmSmem, s>>>(
-        act, 0, 0, 0, nrt, nct, 0, 0, 0, A.p, SA.p, ea.p, ST.p, et.p, D.p, flags);
+        act, 0, 0, 0, nrt, nct, 0, 0, 0, A.p, SA.p, ea.p, ST.p, et.p, D.p, flags, opt.wait_ns);
     MSP_TRY(launch_status());
   }
   unscramble_kernel<<<dim3(div_up(n, 32), div_up(n, 32)), 256, 0, s>>>(n, act, cols_p, A.p, rs.p, cs.p,
@@ -1508,11 +1521,11 @@ int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const d
 }  // namespace msp
 
 // For tests of the variants that a whole GPU or a small matrix never takes: the inverse of a
-// CSR matrix (device arrays) with panels of `cluster` CTAs and at least panel_rows rows a thread.
-// Not part of the interface.
+// CSR matrix (device arrays) with panels of `cluster` CTAs and at least panel_rows rows a thread,
+// and the limit of the products' waits (< 0: the usual one).  Not part of the interface.
 extern "C" int msp_test_inverse(int32_t n, int32_t nnz, const int32_t* d_rp, const int32_t* d_ci,
                                 const double* d_v, double* d_out, int32_t cluster, int32_t panel_rows,
-                                void* stream) {
+                                int64_t wait_ns, void* stream) {
   using namespace msp;
   DevBuf<DevFlags> flags;
   MSP_TRY(flags.alloc(1));
@@ -1520,5 +1533,6 @@ extern "C" int msp_test_inverse(int32_t n, int32_t nnz, const int32_t* d_rp, con
   InverseOptions opt;
   opt.cluster = cluster;
   opt.panel_rows = panel_rows;
+  if (wait_ns >= 0) opt.wait_ns = (unsigned long long)wait_ns;
   return coarse_inverse_blocked(n, nnz, d_rp, d_ci, d_v, d_out, flags.p, (cudaStream_t)stream, opt);
 }

@@ -108,6 +108,8 @@ int launch_bilu_factor(int b, int r0, int r1, const int* rp, const int* ci, cons
 struct InverseOptions {
   int cluster = 0;     // CTAs of the panels' cluster (0: as many as the device places, 16 or 8)
   int panel_rows = 0;  // at least this many rows of the panel a thread (for tests)
+  static constexpr unsigned long long kWaitNs = 2000000000ULL;
+  unsigned long long wait_ns = kWaitNs;  // limit of a wait inside a product (MSP_ERR_TIMEOUT)
 };
 // out (n x n, row-major) = the inverse of a CSR matrix, in FP64 (coarse_inverse.cu);
 // MSP_ERR_SINGULAR_BLOCK where a column has no nonzero pivot.  Synchronises the stream.

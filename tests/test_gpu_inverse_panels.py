@@ -34,14 +34,14 @@ def _system(n, seed):
     return np.array(rp, np.int32), np.concatenate(ci).astype(np.int32), np.concatenate(v)
 
 
-def _inverse(rp, ci, v, cluster, panel_rows):
+def _inverse(rp, ci, v, cluster, panel_rows, wait_ns=-1, status=_native.MSP_OK):
     n = len(rp) - 1
     d = [torch.from_numpy(x).to(DEV) for x in (rp, ci, v)]
     out = torch.empty(n, n, dtype=torch.float64, device=DEV)
     st = _native.lib().msp_test_inverse(C.c_int32(n), C.c_int32(len(ci)), *(C.c_void_p(x.data_ptr()) for x in d),
                                         C.c_void_p(out.data_ptr()), C.c_int32(cluster), C.c_int32(panel_rows),
-                                        C.c_void_p(torch.cuda.current_stream().cuda_stream))
-    assert st == _native.MSP_OK, st
+                                        C.c_int64(wait_ns), C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == status, st
     return out
 
 
@@ -77,3 +77,14 @@ def test_more_rows_than_one_per_thread(n, cluster):
         ag = product(vals.abs(), x.abs() @ product(vals.abs(), x.abs() @ gi.abs()))
         r = gi - product(vals, x @ gi)
         assert bool((r.abs() <= 8.0 * n * 2.0 ** -53 * ag).all())
+
+
+@pytest.mark.parametrize("n", [1, 97, 2111])
+def test_wait_that_runs_out_is_reported(n):
+    """With a limit of 0 every wait of the products gives up at once: the blocks end by
+    themselves, the inverse returns MSP_ERR_TIMEOUT, and the next one is right."""
+    rp, ci, v = _system(n, 5)
+    first = _inverse(rp, ci, v, 0, 0)
+    _inverse(rp, ci, v, 0, 0, wait_ns=0, status=_native.MSP_ERR_TIMEOUT)
+    torch.cuda.synchronize()
+    assert torch.equal(_inverse(rp, ci, v, 0, 0), first)
