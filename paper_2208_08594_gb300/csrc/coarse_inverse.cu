@@ -1338,6 +1338,12 @@ struct SideStream {
 
 }  // namespace
 
+long long inverse_scratch_bytes(long long n) {
+  const long long lda = (n + kP - 1) / kP * kP, rows = (n + kRowTile - 1) / kRowTile * kRowTile;
+  return 8 * (rows * lda + (n + rows) * kP) + rows / kRowTile * kTileA + lda / kColTile * kTileB +
+         4 * (rows + 2 * lda + 6 * n) + 8 * n + kP * kP * 8 + (long long)kKTiles * kTileB + 24 * kP;
+}
+
 int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const double* v, double* out,
                            DevFlags* flags, cudaStream_t s, const InverseOptions& opt) {
   if (n <= 0) return MSP_ERR_ARG;

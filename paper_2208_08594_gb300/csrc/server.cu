@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "setup_kernels.h"
 
 namespace {
 
@@ -343,11 +344,11 @@ int64_t msp_estimate_device_bytes(int32_t nb, int32_t b, int64_t nnzb, const msp
   // level 0: values, BILU factors, stage-N blocks, staging for new values, column 0,
   // pattern and permutations; the pressure matrix and the AMG levels with their ELL
   // copies (at most about 3 nonzeros of pressure per block, both forms); Krylov bases V and
-  // Z and work vectors; the coarsest dense inverse and its panel copy
+  // Z and work vectors; the coarsest dense inverse and what its SETUP works in
   int64_t bytes = nnzb * (3 * bb * 8 + bn * 8 + b * 8 + 16) + (int64_t)nb * (bb * 8 + bn * 8 + 64);
   bytes += nnzb * 3 * (8 + 4) * 2;
   bytes += n * 8 * (2 * (int64_t)m + 16);
-  bytes += nc * nc * 8 * 2;
+  bytes += nc * nc * 8 + msp::inverse_scratch_bytes(nc);
   if (cfg && cfg->precision == MSP_PRECISION_FP32) bytes += nnzb * (2 * bb + bn) * 4;  // FP32 copies
   return bytes + (4ll << 20);
 }

@@ -111,6 +111,9 @@ struct InverseOptions {
   static constexpr unsigned long long kWaitNs = 2000000000ULL;
   unsigned long long wait_ns = kWaitNs;  // limit of a wait inside a product (MSP_ERR_TIMEOUT)
 };
+// device memory that coarse_inverse_blocked allocates and releases for n rows (without the copy
+// of the matrix's nonzeros): the matrix in whole tiles, panels, digits
+long long inverse_scratch_bytes(long long n);
 // out (n x n, row-major) = the inverse of a CSR matrix, in FP64 (coarse_inverse.cu);
 // MSP_ERR_SINGULAR_BLOCK where a column has no nonzero pivot.  Synchronises the stream.
 int coarse_inverse_blocked(int n, int nnz, const int* rp, const int* ci, const double* v, double* out,

@@ -70,3 +70,13 @@ def test_estimate_grows_with_the_system():
     # at least the values, the ILU factors and the Krylov bases
     n = 100000 * 4
     assert big >= 700000 * 16 * 8 * 2 + n * 8 * 2 * 30
+
+
+def test_estimate_holds_the_scratch_of_the_coarsest_inverse():
+    """The coarsest level of 10,000 rows: its inverse, and during SETUP the matrix in whole tiles
+    of 128 rows and panels of 96 columns, two panels, and the digits of one step (16 bytes per
+    operand: eight of bf16), of rows and of columns."""
+    from paper_2208_08594_gb300 import _native
+    n, rows, cols = 10000, 10112, 10080
+    need = 8 * n * n + 8 * rows * cols + 2 * 8 * 96 * n + 16 * 96 * (rows + cols)
+    assert _native.msp_estimate_device_bytes(n, 1, 7 * n) >= need
