@@ -34,12 +34,11 @@ int launch_bsr_spmv_perm(int b, int nb, const int* rp, const int* ci, const doub
                          const int* perm, const double* x, double* y, cudaStream_t s,
                          LongRows lr);
 // rP[i] = omega_i^T (g_i - (A w)_i)   (omega == nullptr: first unknown only); r != nullptr
-// also receives g - A w.  after_n (with r): the pressure slots of w are zero (stage N)
+// also receives g - A w, and the pressure slots of w must be zero (as stage N leaves them)
 template <typename T>
 int launch_bsr_restrict_p(int b, int nb, const int* rp, const int* ci, const T* v, const T* w,
-                          const T* g, const T* omega, T* rP, T* r, bool after_n,
-                          cudaStream_t s, const unsigned char* rmask = nullptr,
-                          LongRows lr = LongRows());
+                          const T* g, const T* omega, T* rP, T* r, cudaStream_t s,
+                          const unsigned char* rmask = nullptr, LongRows lr = LongRows());
 // r_i <- r_i - sum_j A_ij[:, 0] e_j and w_i[0] += e_i (r, w: nb*b values; c0: column 0 of
 // every block, nnzb*b values; e: one value per block row)
 template <typename T>

@@ -1359,14 +1359,15 @@ inline double bsr_bytes(msp_handle h, double sT, double vecs) {
 
 template <typename T>
 int stage_P(msp_handle h, const PView<T>& P, const T* g, T* w, T* r, cudaStream_t s) {
-  // r != nullptr: leave in r the residual g - A w of the corrected w (stage R's input),
+  // r != nullptr (w is stage N's, its pressure slots zero): leave in r the residual g - A w of
+  // the corrected w (stage R's input),
   // as (g - A w_before) - A Pi_P e instead of a second pass over the whole matrix
   const double sT = sizeof(T), b = h->b;
   {
     Probe pr("stageP_residual_restrict", bsr_bytes(h, sT, r ? 3 : 2) + (double)h->nb * sT, s,
              1, sT == 8 ? 2.0 * (bsr_fmas(h) + (double)h->nb * b) : 0.0);
     MSP_TRY(launch_bsr_restrict_p<T>(h->b, h->nb, h->rp.p, h->ci.p, P.vals, w, g, P.omega,
-                                     P.lb[0], r, true, s, P.m0, long_rows(h, 0, h->nb)));
+                                     P.lb[0], r, s, P.m0, long_rows(h, 0, h->nb)));
   }
   MSP_TRY(vcycle<T>(h, P, 0, s));
   if (!r) {

@@ -336,13 +336,13 @@ __global__ void __launch_bounds__(kThreads) bsr_spmv_kernel(int nb, const int* _
 }
 
 // ----------------------------------------------------------------------------------
-// rP[i] = omega_i^T (g_i - (A w)_i); with WR the residual g - A w is also stored in r
-// AFTERN: w comes from stage N, so its pressure slots are zero and column 0 of the blocks is
-// not multiplied (the FP64 FMAs bound the kernel: 1.12M x 4 242 -> 198 us, 132k x 4 38 ->
+// rP[i] = omega_i^T (g_i - (A w)_i); with WR the residual g - A w is also stored in r, and w
+// comes from stage N, so its pressure slots are zero and column 0 of the blocks is not
+// multiplied (the FP64 FMAs bound the kernel: 1.12M x 4 242 -> 198 us, 132k x 4 38 ->
 // 33 us).  The concentration rows of the last
 // colour are not zero in general: the matrix may be newer than the preconditioner.
 // ----------------------------------------------------------------------------------
-template <int B, typename T, bool WR, bool AFTERN>
+template <int B, typename T, bool WR>
 __global__ void __launch_bounds__(kThreads) bsr_restrict_p_kernel(
     int nb, const int* __restrict__ rp, const int* __restrict__ ci, const T* __restrict__ v,
     const T* __restrict__ w, const T* __restrict__ g, const T* __restrict__ omega,
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kThreads) bsr_restrict_p_kernel(
     for (int k = 1; k < B; ++k) res += __shfl_sync(0xffffffffu, term, k);
     if (l == 0) rP[i] = res;
   }
-  constexpr int GP = Gp<B>::v, kFirst = AFTERN ? 1 : 0;  // first column multiplied
+  constexpr int GP = Gp<B>::v, kFirst = WR ? 1 : 0;  // first column multiplied
   const int lane = threadIdx.x % GP;
   const int gpb = blockDim.x / GP;
   // the loop bound depends on the block only, so every lane reaches the group shuffle
@@ -1790,19 +1790,16 @@ int launch_bsr_spmv_perm(int b, int nb, const int* rp, const int* ci, const doub
 
 template <typename T>
 int launch_bsr_restrict_p(int b, int nb, const int* rp, const int* ci, const T* v, const T* w,
-                          const T* g, const T* omega, T* rP, T* r, bool after_n,
-                          cudaStream_t s, const unsigned char* rmask, LongRows lr) {
+                          const T* g, const T* omega, T* rP, T* r, cudaStream_t s,
+                          const unsigned char* rmask, LongRows lr) {
   if (nb <= 0) return MSP_OK;
   MSP_B_SWITCH(b, {
     const unsigned grid = with_long_rows(grid_groups(nb, Gp<B_>::v), lr.n);
-    if (r && after_n)
-      bsr_restrict_p_kernel<B_, T, true, true><<<grid, kThreads, 0, s>>>(
-          nb, rp, ci, v, w, g, omega, rP, r, rmask, lr.rows, lr.n, lr.thr);
-    else if (r)
-      bsr_restrict_p_kernel<B_, T, true, false><<<grid, kThreads, 0, s>>>(
+    if (r)
+      bsr_restrict_p_kernel<B_, T, true><<<grid, kThreads, 0, s>>>(
           nb, rp, ci, v, w, g, omega, rP, r, rmask, lr.rows, lr.n, lr.thr);
     else
-      bsr_restrict_p_kernel<B_, T, false, false><<<grid, kThreads, 0, s>>>(
+      bsr_restrict_p_kernel<B_, T, false><<<grid, kThreads, 0, s>>>(
           nb, rp, ci, v, w, g, omega, rP, r, rmask, lr.rows, lr.n, lr.thr);
   });
   return launch_status();
@@ -2339,8 +2336,8 @@ int launch_scatter_blocks(int nb, int b, const int* perm, const double* in, doub
                                   const T*, T*, bool, cudaStream_t, const unsigned char*,   \
                                   LongRows);                                                \
   template int launch_bsr_restrict_p<T>(int, int, const int*, const int*, const T*,         \
-                                        const T*, const T*, const T*, T*, T*, bool,         \
-                                        cudaStream_t, const unsigned char*, LongRows); \
+                                        const T*, const T*, const T*, T*, T*, cudaStream_t, \
+                                        const unsigned char*, LongRows);                    \
   template int launch_bsr_col0_update<T>(int, int, const int*, const int*, const T*,        \
                                          const T*, T*, T*, cudaStream_t, const unsigned char*, \
                                          LongRows);                                          \
