@@ -305,9 +305,9 @@ __global__ void segment_sums_kernel(int nseg, const int* __restrict__ seg_start,
 // the smallest index among equals) is simply the smallest label.  V of the current pass and
 // the frontier hat W (always a subset of V: a vertex leaving V leaves the frontier too, where
 // the else branch of Algorithm 4.1 would only move it to Wbar, where it already is) are
-// bitmaps; the Wbar list of a pass is V of the next one.  The frontier has two summary
-// levels above its words, whose bits may be stale (set for an empty word) and are corrected
-// when a search meets them, so that clearing a bit touches one word.  The next pick is the
+// bitmaps; the Wbar list of a pass is V of the next one.  The frontier has one summary above
+// its words, a bit per 32 words (1024 labels), which may be stale (set over empty words) and is
+// corrected when a search meets it, so that clearing a bit touches one word.  The next pick is the
 // frontier's first bit; with an empty frontier the smallest label still in V (a cursor that
 // only moves forward).
 //
@@ -342,13 +342,11 @@ __global__ void __launch_bounds__(32 * kBatch) colouring_batch_kernel(
   __shared__ int before[32];  // frontier vertices before each word of the candidates' group
   __shared__ int s_nc, s_group, s_nwbar;
   const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
-  const int n0 = (n + 31) / 32, n1 = (n0 + 31) / 32, n2 = (n1 + 31) / 32;
+  const int n0 = (n + 31) / 32, n2 = (n + 32767) / 32768;
   volatile unsigned* l2 = smem_bits;
-  volatile unsigned* l1 = smem_bits + n2;
-  unsigned* V = VS ? smem_bits + n2 + n1 : gV;
-  unsigned* F = FS ? smem_bits + n2 + n1 + (VS ? n0 : 0) : gF;
+  unsigned* V = VS ? smem_bits + n2 : gV;
+  unsigned* F = FS ? smem_bits + n2 + (VS ? n0 : 0) : gF;
   for (int k = threadIdx.x; k < n2; k += 32 * kBatch) l2[k] = 0u;
-  for (int k = threadIdx.x; k < n1; k += 32 * kBatch) l1[k] = 0u;
   for (int k = threadIdx.x; k < n0; k += 32 * kBatch) {
     const int rem = n - 32 * k;
     F[k] = 0u;
@@ -388,10 +386,7 @@ __global__ void __launch_bounds__(32 * kBatch) colouring_batch_kernel(
           unsigned w = wi < n0 ? *(volatile unsigned*)(F + wi) : 0u;
           const unsigned m = __ballot_sync(kAll, w != 0u);
           __syncwarp();
-          if (lane == 0) {
-            l1[i1] = m;
-            if (m == 0u) l2[i2] = l2[i2] & ~(1u << (i1 & 31));
-          }
+          if (lane == 0 && m == 0u) l2[i2] = l2[i2] & ~(1u << (i1 & 31));
           __syncwarp();
           if (m == 0u) continue;
           const int cnt = __popc(w);
@@ -530,7 +525,6 @@ __global__ void __launch_bounds__(32 * kBatch) colouring_batch_kernel(
         auto join = [&](int y) {
           if (!((v_word(y) >> (y & 31)) & 1u)) return;
           atomicOr(F + (y >> 5), 1u << (y & 31));
-          atomicOr((unsigned*)l1 + (y >> 10), 1u << ((y >> 5) & 31));
           atomicOr((unsigned*)l2 + (y >> 15), 1u << ((y >> 10) & 31));
           // the next picks come from here: their list's place is then an L1 hit
           asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(meta + y)));
@@ -557,7 +551,7 @@ __global__ void __launch_bounds__(32 * kBatch) colouring_batch_kernel(
 // The same one pick at a time, the second circle gathered from the neighbours' rows (every
 // lane issuing its loads back to back, owner rows looked up in shared memory): for callers
 // without room for lists, graphs whose lists would not fit 32-bit offsets (a vertex joined
-// to most of a large graph) and more labels than the batched kernel keeps summaries of.
+// to most of a large graph) and more labels than colouring_batch_ok takes.
 constexpr size_t kColouringSmem = 220 * 1024;
 
 struct Bitmap3 {
@@ -1002,10 +996,8 @@ int launch_colouring(int n, const int* srp, const int* sci, unsigned* inV, int* 
   return launch_status();
 }
 
-bool colouring_batch_ok(int n) {
-  const size_t n1 = ((size_t)n + 1023) / 1024, n2 = (n1 + 31) / 32;
-  return (n1 + n2) * sizeof(unsigned) <= 64 * 1024;
-}
+// a search reads the whole summary (2 kB at the limit); larger graphs were not measured
+bool colouring_batch_ok(int n) { return n <= 1 << 24; }
 
 int launch_colouring_batch(int n, const int4* lists, const int* list, unsigned* inV, int* wbar,
                            unsigned* bitmap, int* colour, int* meta, int max_passes,
@@ -1013,7 +1005,7 @@ int launch_colouring_batch(int n, const int4* lists, const int* list, unsigned* 
   if (n <= 0) return MSP_OK;
   if (!colouring_batch_ok(n)) return MSP_ERR_ARG;
   const size_t w0 = sizeof(unsigned) * (((size_t)n + 31) / 32);
-  const size_t n1 = ((size_t)n + 1023) / 1024, sum = sizeof(unsigned) * (n1 + (n1 + 31) / 32);
+  const size_t sum = sizeof(unsigned) * (((size_t)n + 32767) / 32768);
   // V is read most, then the frontier's words
   auto run = [&](auto kern, size_t smem) -> int {
     MSP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
