@@ -1038,7 +1038,10 @@ PView<float> view32(msp_handle h) {
 
 // Whether the residual restriction of a level of n rows reads only the entries right of the
 // diagonal (after one forward colour sweep from zero the others cancel): on levels bound
-// by bandwidth.
+// by bandwidth.  Applications in us with it on level 0 / with whole rows (b = 4, FP64; FP32):
+// 35k rows 428 / 426; 371 / 367, 200k 756 / 756; 512 / 510, 328k 995 / 998; 700 / 702, 554k
+// 1428 / 1426; 959 / 969, 818k 1828 / 1838; 1229 / 1225, 1.12M 2329 / 2336; 1530 / 1536: a loss
+// on small levels, a gain of 0.3 to 0.5 % on the largest, neither within 1 % in between.
 bool restrict_upper(msp_handle h, int n) {
   return h->cfg.smoother == MSP_SMOOTHER_PGS_MC && h->cfg.pre_sweeps == 1 && n > 262144;
 }

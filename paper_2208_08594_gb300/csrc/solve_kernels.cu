@@ -819,8 +819,8 @@ __global__ void __launch_bounds__(kThreads) ell_gs_colour_kernel(
 // UPPER (after one forward sweep from zero): a row was solved with the values of the earlier
 // colours and zeros for the later ones, so b_i - (A x)_i is minus its entries right of the
 // diagonal times x, and only those are read, once meta is there.  For levels bound by
-// bandwidth (1.12M rows: 57.6 -> 45.8 us); on small ones the further trip to memory costs more
-// (132k-row application 458 against 476 us with it everywhere).
+// bandwidth (1.12M rows: 57.6 -> 45.8 us); on small ones the further trip to memory costs as
+// much or more (see restrict_upper).
 template <typename T, int K, int TPR, bool UPPER>
 __global__ void __launch_bounds__(kThreads) ell_residual_restrict_kernel(
     int nc, const int* __restrict__ mptr, const int* __restrict__ members,
@@ -1829,6 +1829,10 @@ int launch_extract_col0(size_t nnzb, int b, const T* v, T* c0, cudaStream_t s) {
 // one: classes of a few blocks, whose time is the chain of loads that then overlaps the
 // previous launch.  A class that fills the SMs only holds places with waiting blocks: with a
 // limit of 600k threads the 132k-row application lost 2 % (b = 4, 66k rows a class).
+// Applications in us with no dependent classes / this limit / 20,000 / 50,000 / 200,000: 2k
+// cells, b = 3: 211 / 193 / 192 / 195 / 192; 9.5k, b = 6: 485 / 433 / 379 / 379 / 382; 30k,
+// b = 6: 558 / 515 / 496 / 530 / 517; 70k, b = 4: 490 / 478 / 479 / 468 / 489.  So this limit is
+// on the safe side of where the gain ends (20,000 to 50,000, by the block size).
 constexpr size_t kBgsPdlThreads = 8192;
 
 template <typename T>
