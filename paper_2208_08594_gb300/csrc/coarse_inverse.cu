@@ -787,20 +787,18 @@ __device__ __forceinline__ void tmem_ld8(unsigned addr, unsigned (&r)[8]) {
       : "r"(addr));
 }
 
-// c + 2^(e + 16) sum_m S_m 2^(8 (5 - m)), m = 0..5, S_m exact integers below 2^24 (as below,
-// with two words of three digits)
+// c + 2^(e + 16) sum_m S_m 2^(8 (5 - m)), m = 0..5, |S_m| <= (m + 1) 2^21: an integer below 2^62,
+// taken without its last 12 bits (2^-49 of the largest product, as the digits left out) so that it
+// becomes a double by one subtraction: two FP64 operations an element
 __device__ __forceinline__ double add_digits(const float (&S)[6], int e, double, double c) {
+  static_assert(CorrGeo::kK << 14 <= 1 << 21, "bound of the sums");
   const int s0 = __float2int_rn(S[0]), s1 = __float2int_rn(S[1]), s2 = __float2int_rn(S[2]);
   const int s3 = __float2int_rn(S[3]), s4 = __float2int_rn(S[4]), s5 = __float2int_rn(S[5]);
-  const long long hi = (long long)s0 * 65536 + ((long long)s1 * 256 + s2);
-  const long long lo = (long long)s3 * 65536 + ((long long)s4 * 256 + s5);
-  // M = 1.5 * 2^52 = 1.5 * 2^28 * 2^24
-  const double dh =
-      __longlong_as_double(0x4338000000000000LL + (hi - 402653184)) - 6755399441055744.0;
-  const double dl = __longlong_as_double(0x4338000000000000LL + lo);
-  const int be = min(max(e + 1039, 0), 0x7ff), bh = min(max(e + 1063, 0), 0x7ff);
-  return fma(dl, __longlong_as_double((long long)be << 52),
-             fma(dh, __longlong_as_double((long long)bh << 52), c));
+  const long long v = (long long)(s0 * 256 + s1) * 1048576 + (long long)(s2 * 256 + s3) * 16 +
+                      ((s4 + (s5 >> 8) + 8) >> 4);
+  const double d = __longlong_as_double(0x4338000000000000LL + v) - 6755399441055744.0;
+  const int be = min(max(e + 1051, 0), 0x7ff);
+  return fma(d, __longlong_as_double((long long)be << 52), c);
 }
 // c + sign 2^e sum_m S_m 2^(8 (7 - m)), m = 0..7, S_m exact integers below 2^24
 __device__ __forceinline__ double add_digits(const float (&S)[8], int e, double sign, double c) {
