@@ -1274,15 +1274,18 @@ int vcycle(msp_handle h, const PView<T>& P, int l, cudaStream_t s) {
     MSP_TRY(phase(order, true));
   }
   {
+    // with the entries right of the diagonal alone neither b nor the diagonal is read
+    const bool upper = L.ell_k > 0 && restrict_upper(h, n);
     const double bytes =
-        (double)L.A.nnz * (sT + 4) + (double)n * (3 * sT + 12) + (double)L.nc * (sT + 4);
+        (upper ? 0.5 * (double)(L.A.nnz - n) * (sT + 4) + (double)n * (sT + 8)
+               : (double)L.A.nnz * (sT + 4) + (double)n * (3 * sT + 12)) +
+        (double)L.nc * (sT + 4);
     if (L.ell_k > 0) {
       Probe pr(level_site("amg_residual_restrict_l", l), bytes, s);
       MSP_TRY(launch_ell_residual_restrict<T>(L.ell_k, L.nc, L.mptr.p, L.members.p, L.ell_ci.p,
                                               P.lev[l], L.ell_meta.p, P.led[l], L.A.rp.p,
                                               L.A.ci.p, P.lv[l], L.dpos.p, P.lb[l], P.lx[l],
-                                              P.lb[l + 1], s, P.lm[l + 1], L.rr_tpr,
-                                              restrict_upper(h, n)));
+                                              P.lb[l + 1], s, P.lm[l + 1], L.rr_tpr, upper));
     } else {
       Probe pr(level_site("amg_residual_restrict_csr_l", l), bytes, s);
       MSP_TRY(launch_csr_residual_restrict<T>(L.nc, L.mptr.p, L.members.p, L.A.rp.p,
@@ -1368,7 +1371,7 @@ int stage_P(msp_handle h, const PView<T>& P, const T* g, T* w, T* r, cudaStream_
   const double sT = sizeof(T), b = h->b;
   {
     Probe pr("stageP_residual_restrict", bsr_bytes(h, sT, r ? 3 : 2) + (double)h->nb * sT, s,
-             1, sT == 8 ? 2.0 * (bsr_fmas(h) + (double)h->nb * b) : 0.0);
+             1, sT == 8 ? 2.0 * (bsr_fmas(h) * (r ? (b - 1) / b : 1.0) + (double)h->nb * b) : 0.0);
     MSP_TRY(launch_bsr_restrict_p<T>(h->b, h->nb, h->rp.p, h->ci.p, P.vals, w, g, P.omega,
                                      P.lb[0], r, s, P.m0, long_rows(h, 0, h->nb)));
   }
