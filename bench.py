@@ -294,10 +294,12 @@ def kernel_source_sha(kernel):
     return None
 
 
-def traffic_for(kernel):
+def traffic_for(kernel, precision="fp64", dims=(60, 220, 85)):
     """DRAM bytes (read + write) per launch of `kernel` at the benchmark size, from the
-    committed ncu summary, if it was taken on the current source of that kernel (null
-    otherwise)."""
+    committed ncu summary, if it was taken on the current source of that kernel and in this
+    precision and size (null otherwise: the summary is FP64 at 60x220x85)."""
+    if precision != "fp64" or tuple(dims) != (60, 220, 85):
+        return None
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as f:
@@ -570,7 +572,7 @@ def run_native(args):
         name, rec = max(kern.items(), key=lambda kv: kv[1][1])
         roofline = roofline_of(name, rec, peak, peak_kind, sms, sm_mhz, fma64, live_ms,
                                args.steps)
-        roofline.update({"traffic": traffic_for(name),
+        roofline.update({"traffic": traffic_for(name, args.precision, (args.nx, args.ny, args.nz)),
                     "measured": "CUDA event pairs around every call site (one launch, or "
                                 "the consecutive launches of one kernel over the colours of "
                                 "a sweep), as event nodes inside the preconditioner's CUDA "

@@ -107,3 +107,11 @@ def test_reference_arm_prints_the_contract_line_on_rank_0_only():
                            "d2h_bytes_per_step": 0}
     assert line["config"]["cells"] == 120
     assert _bench(args, env={"RANK": "1", "WORLD_SIZE": "2"}) == []
+
+
+def test_traffic_is_that_of_the_captured_precision_and_size():
+    """The committed DRAM traffic is FP64 at 60x220x85: no other run may report it."""
+    for k in ("bgs_colour_kernel", "bsr_spmv_kernel"):
+        assert bench.traffic_for(k) == bench.traffic_for(k, "fp64", (60, 220, 85))
+        assert bench.traffic_for(k, "fp32", (60, 220, 85)) is None
+        assert bench.traffic_for(k, "fp64", (30, 110, 42)) is None
