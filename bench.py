@@ -572,7 +572,9 @@ def run_native(args):
         name, rec = max(kern.items(), key=lambda kv: kv[1][1])
         roofline = roofline_of(name, rec, peak, peak_kind, sms, sm_mhz, fma64, live_ms,
                                args.steps)
-        roofline.update({"traffic": traffic_for(name, args.precision, (args.nx, args.ny, args.nz)),
+        roofline.update({"traffic": traffic_for(
+                             name, args.precision if args.wells == "rows" and args.colouring == "alg41"
+                             else None, (args.nx, args.ny, args.nz)),
                     "measured": "CUDA event pairs around every call site (one launch, or "
                                 "the consecutive launches of one kernel over the colours of "
                                 "a sweep), as event nodes inside the preconditioner's CUDA "

@@ -21,26 +21,25 @@
 // the digits 1..9-i of T side by side (N = 32 (9 - i)), each into the accumulator columns of its
 // i + j.
 //
-// Such a product is exact to about 2^-56 of the row's times the column's largest operand: as an
-// FP64 product in norm, but its small entries lose what FP64 products of small operands keep,
-// and where rows of A are in other units than the rest that reaches the large entries (four
-// rows times 1e10: 2e-9 of the largest entry; FP64 elimination 5e-15).  Hence the scaling, and
-// after the elimination one step X += X (I - B X): the residual in FP64 from the sparse matrix B,
-// the product in six digits of the already small term (four left entries of 1e-14 of the largest
-// with fewer correct digits than FP64 elimination where the permeability spans e^(4N)).
-// Errors of the algorithm against an extended-precision inverse, with FP64 elimination in
-// parentheses, as a fraction of the largest entry and of the entry itself: coarsest level of 742
-// rows 1.7e-16 (8.2e-16) and 3.5e-13 (9.4e-13); permeabilities e^(4N) 7.5e-15 (1.1e-14) and
-// 5.2e-13 (2.4e-11); rows times 10^U[-9,9] 9e-17 (1e-11) and 7e-16 (7e-6); elimination with an
-// exchange in every column, 1,000 rows, 1.1e-14 (1.5e-13) and 6e-10 (1.6e-8).
+// Such a product errs by about 2^-56 of its row's times its column's largest operand: as an
+// FP64 product in norm, but operands below 2^-10 of their row's or column's maximum keep fewer
+// than 53 bits, so small entries of the inverse lose digits (5e-9 to 2e-7 of themselves), and
+// where rows of A are in other units than the rest so do the large ones (four rows times 1e10:
+// 2e-9 of the largest entry; FP64 elimination 7e-16).  Hence the scaling, and after the
+// elimination one step X += X (I - B X): the residual in FP64 from the sparse matrix B, the
+// product in six digits of the already small term.  Errors against an extended-precision
+// inverse, digits alone / now / FP64 elimination, as a fraction of the largest entry and of the
+// entry itself (emulated): coarsest level of 742 rows 2e-16 / 3e-16 / 8e-16 and 8e-9 / 4e-13 /
+// 9e-13; permeabilities e^(4N) 9e-15 / 6e-15 / 1e-14 and 2e-7 / 4e-13 / 2e-11; rows times
+// 10^U[-9,9] 4e-3 / 9e-17 / 1e-11 and 7e3 / 9e-16 / 7e-6; an exchange in every column, 1,000 rows,
+// 3e-15 / 1e-14 / 2e-13 and 4e-9 / 2e-9 / 2e-8.
 //
-// One SETUP's inverse, before (rank-32 updates on the FP64 pipes, two launches per column)
-// and now: n = 2,048: 45 -> 13 ms, 4,231: 203 -> 30 ms, 5,867: 446 -> 46 ms, 9,836: 1,824 ->
-// 109 to 135 ms (14 to 17 FP64 TFLOP/s, as the panels' clusters find their place).  Errors against an extended-precision solve are below the
-// previous kernels' (9,836 rows: 7.5e-16 against 1.8e-15).  What bounds it: the panels'
-// columns (3.5 us each, a chain of one cluster exchange, a reciprocal and the rank-1
-// update) up to about 6,000 rows, above that the products, whose epilogue keeps the FP64
-// pipe and the trips to TMEM and memory busy (tensor pipe 25 %).
+// One SETUP's inverse, with rank-32 updates on the FP64 pipes (two launches per column) and now:
+// n = 2,048: 45 -> 14.5 ms, 4,231: 203 -> 36.5 ms, 5,867: 446 -> 60 ms, 9,836: 1,824 -> 164 ms; of
+// it the correction 1, 6.5, 14 and 55 ms.  What bounds it: the panels' columns (3.5 us each, a
+// chain of one cluster exchange, a reciprocal and the rank-1 update) up to about 6,000 rows,
+// above that the products, a tile's chain of MMAs and an epilogue that keeps the FP64 pipe half
+// busy (tensor pipe 19 to 28 %).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
