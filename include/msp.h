@@ -61,7 +61,8 @@ extern "C" {
 
 /* Arithmetic of the preconditioner (msp_config.precision).  FGMRES, its residuals,
  * orthogonalisation and Hessenberg least squares, and the coarsest dense solve are
- * always FP64. */
+ * always FP64 (the inverse it applies is formed on the tensor cores, with errors no larger
+ * than those of elimination in FP64). */
 #define MSP_PRECISION_FP64 0
 #define MSP_PRECISION_FP32 1 /* stage N/P/R values and arithmetic in FP32 */
 
